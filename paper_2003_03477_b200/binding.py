@@ -27,7 +27,7 @@ SS_SYNC_BMUF_NESTEROV = 2
 
 EXPORTS = ["ss_status_str", "ss_last_cuda_error", "ss_num_sms", "ss_embbag_fwd", "ss_embbag_bwd_workspace_bytes",
            "ss_embbag_bwd_adagrad", "ss_embbag_bwd_sort", "ss_embbag_bwd_apply", "ss_embbag_bwd_sort_noalloc", "ss_mlp_param_count", "ss_mlp_param_offsets", "ss_mlp_workspace_bytes",
-           "ss_mlp_fwd", "ss_mlp_bwd", "ss_train_step", "ss_ne_accumulate", "ss_ne_value", "ss_sync_easgd", "ss_sync_ma", "ss_sync_bmuf", "ss_shadow_start", "ss_shadow_rounds", "ss_shadow_pause", "ss_shadow_stop", "ss_to_bf16",
+           "ss_mlp_fwd", "ss_mlp_bwd", "ss_train_step", "ss_step_plan_create", "ss_step_plan_destroy", "ss_step_plan_counts", "ss_ne_accumulate", "ss_ne_value", "ss_sync_easgd", "ss_sync_ma", "ss_sync_bmuf", "ss_shadow_start", "ss_shadow_rounds", "ss_shadow_pause", "ss_shadow_stop", "ss_to_bf16",
            "ss_gemm_bf16", "ss_device_error", "ss_mlp_set_flow_ctas", "ssh_fill_uniform", "ss_profile", "ss_profile_collect"]
 
 
@@ -78,6 +78,9 @@ def lib() -> C.CDLL:
         L.ss_mlp_fwd.argtypes = [C.POINTER(MlpDesc), vp, vp, vp, vp, vp, i32, vp, vp, vp, vp, vp, sz, vp]
         L.ss_mlp_bwd.argtypes = [C.POINTER(MlpDesc), vp, vp, vp, vp, vp, vp, vp, vp, vp, i32, f32, f32, i32,
                                  vp, i64, vp, sz, vp]
+        L.ss_step_plan_create.argtypes = [C.POINTER(vp)]
+        L.ss_step_plan_destroy.argtypes = [vp]
+        L.ss_step_plan_counts.argtypes = [vp, C.POINTER(i64)]
         L.ss_ne_accumulate.argtypes = [vp, vp, i32, vp, vp]
         L.ss_ne_value.argtypes = [vp, vp, vp]
         L.ss_sync_easgd.argtypes = [C.POINTER(vp), i32, vp, i64, f32, i32, C.POINTER(vp), vp]
@@ -101,6 +104,7 @@ def lib() -> C.CDLL:
             if name not in ("ss_status_str", "ss_last_cuda_error", "ss_num_sms", "ss_embbag_bwd_workspace_bytes",
                             "ss_mlp_param_count", "ss_mlp_workspace_bytes", "ss_shadow_rounds", "ss_mlp_set_flow_ctas"):
                 getattr(L, name).restype = i32
+        L.ss_step_plan_destroy.restype = None
         _lib = L
     return _lib
 
@@ -254,13 +258,36 @@ def ss_mlp_bwd(spec: MlpSpec, w, w_bf16, adagrad_acc, grads, dense, concat_f32, 
 
 def ss_train_step(spec: MlpSpec, tables, row_state, T, N, D, B, indices, offsets, L, dense, labels, w, w_bf16, adagrad_acc,
                   concat_f32, concat_bf16, logit, prob, loss, grad_pooled, mlp_ws, emb_ws, uniq_keys, seg_off, perm,
-                  d_num_unique, d_status, lr, eps, replicas, stream, sort_stream, mlp_stream) -> None:
+                  d_num_unique, d_status, lr, eps, replicas, stream, sort_stream, mlp_stream,
+                  plan: Optional["StepPlan"] = None) -> None:
     st = native().ss_train_step(spec.desc_address, tables, row_state, T, N, D, B, indices, offsets, L, dense, labels, w,
                                 w_bf16, adagrad_acc, concat_f32, concat_bf16, logit, prob, loss, grad_pooled, mlp_ws,
                                 emb_ws, uniq_keys, seg_off, perm, d_num_unique, d_status, lr, eps, replicas, stream,
-                                sort_stream, mlp_stream)
+                                sort_stream, mlp_stream, None if plan is None else plan.handle)
     if st:
         _check("ss_train_step", st)
+
+
+class StepPlan:
+    """What ss_train_step keeps for one training loop (ss_step_plan): the step as a CUDA graph, freed with the object."""
+
+    handle = None
+
+    def __init__(self):
+        h = C.c_void_p()
+        _check("ss_step_plan_create", lib().ss_step_plan_create(C.byref(h)))
+        self.handle = h.value
+
+    def counts(self):
+        """(steps enqueued directly, steps launched as a graph, graph nodes updated, graphs held)"""
+        c = (C.c_int64 * 4)()
+        _check("ss_step_plan_counts", lib().ss_step_plan_counts(self.handle, c))
+        return tuple(c)
+
+    def __del__(self):
+        if self.handle is not None and _lib is not None:
+            _lib.ss_step_plan_destroy(self.handle)
+            self.handle = None
 
 
 def ss_ne_accumulate(logit, labels, B, acc, stream=None) -> None:

@@ -1,8 +1,10 @@
-// Status strings, device checks, float->bf16 conversion.
+// Status strings, device checks, launches, float->bf16 conversion.
 #include "common.cuh"
+#include "profile.cuh"
 
 namespace ss {
 thread_local int g_last_cuda_error = 0;
+thread_local StepSink* g_step_sink = nullptr;
 
 static int g_arch_ok[64];   // 0 unknown, 1 ok, -1 not sm_100
 static int g_sms[64];
@@ -26,6 +28,30 @@ int num_sms() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
   if (g_arch_ok[dev] == 0) check_arch();
   return g_sms[dev] > 0 ? g_sms[dev] : 148;
+}
+
+cudaError_t launch_now(const LaunchShape& shape, cudaStream_t st, void** params) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = shape.grid; cfg.blockDim = shape.block; cfg.dynamicSmemBytes = shape.smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)shape.cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = shape.cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelExC(&cfg, shape.kernel, params);
+}
+
+__global__ void clear_words_kernel(int* p, int n) {
+  wait_for_previous_kernel();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0;
+}
+ss_status clear_words(int* p, int n, cudaStream_t st) {
+  SS_TIMED("clear_words_kernel", st);
+  launch_dependent(clear_words_kernel, 1, n < 1024 ? 128 : 1024, 0, st, p, n);
+  SS_LAUNCH_OK();
+  return SS_OK;
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, int64_t n) {

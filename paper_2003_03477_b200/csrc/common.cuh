@@ -32,6 +32,26 @@ inline ss_status cuda_fail(cudaError_t e) {
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline cudaStream_t as_stream(ss_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// What the calls of a training step enqueue.  While a step plan records a step or brings its graph up to date with one
+// (step.cu), their kernels and events go to it; otherwise g_step_sink is null and they go to the streams.
+struct LaunchShape {
+  const void* kernel;
+  dim3 grid, block;
+  size_t smem;
+  int cluster;
+};
+struct StepSink {
+  virtual cudaError_t kernel(const LaunchShape& shape, cudaStream_t st, void** params, const size_t* sizes, int n) = 0;
+  virtual cudaError_t record(cudaEvent_t e, cudaStream_t st) = 0;
+  virtual cudaError_t wait(cudaStream_t st, cudaEvent_t e) = 0;
+ protected:
+  ~StepSink() = default;
+};
+extern thread_local StepSink* g_step_sink;
+cudaError_t launch_now(const LaunchShape& shape, cudaStream_t st, void** params);   // a programmatic dependent launch
+inline cudaError_t step_record(cudaEvent_t e, cudaStream_t st) { return g_step_sink ? g_step_sink->record(e, st) : cudaEventRecord(e, st); }
+inline cudaError_t step_wait(cudaStream_t st, cudaEvent_t e) { return g_step_sink ? g_step_sink->wait(st, e) : cudaStreamWaitEvent(st, e, 0); }
+
 #ifdef __CUDACC__
 // Two independent fused multiply-adds in one instruction (sm_100); each rounds like fmaf.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
@@ -48,18 +68,16 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 // and waits, as the first thing every one of its threads does, until that kernel is complete and its stores are visible.
 // The gap between dependent kernels of a few microseconds all but closes (from about 2.4 us).
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P>
+inline cudaError_t launch_params(const LaunchShape& shape, cudaStream_t st, const P&... args) {
+  void* ptr[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  const size_t size[] = {sizeof(P)...};
+  return g_step_sink ? g_step_sink->kernel(shape, st, ptr, size, (int)sizeof...(P)) : launch_now(shape, st, ptr);
+}
 template <typename... P, typename... A>
 inline cudaError_t launch_cluster_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st, A&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  const LaunchShape shape{reinterpret_cast<const void*>(kernel), grid, block, smem, cluster};
+  return launch_params<P...>(shape, st, std::forward<A>(args)...);
 }
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
@@ -70,5 +88,9 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block,
 // SS_OK when the current device is compute capability 10.x, cached per device.
 ss_status check_arch();
 int num_sms();
+
+// Sets n words to zero by a kernel of one block: it starts as the kernel before it ends, and the next one as it ends (a
+// memset would break that chain).
+ss_status clear_words(int* p, int n, cudaStream_t st);
 
 }  // namespace ss

@@ -1465,11 +1465,6 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, cons
     else { CALL(32, 8); }                                                         \
   } while (0)
 
-__global__ void clear_words_kernel(int* p, int n) {
-  wait_for_previous_kernel();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0;
-}
-
 // Closes an empty sort.
 __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_for_previous_kernel(); finish_unique(o, 0u); }
 
@@ -1619,15 +1614,11 @@ static ss_status bwd_impl(bool do_sort, bool do_apply, float* tables, float* row
     ts.hist = reinterpret_cast<uint32_t*>(ws + p.off_hist); ts.bintot = reinterpret_cast<uint32_t*>(ws + p.off_bintot);
     ts.tile_heads = reinterpret_cast<uint32_t*>(ws + p.off_heads);
     ts.ctl = ctl + kCtlTiled; ts.passes = p.passes; ts.digit_bits = p.digit_bits; ts.bins = p.bins; ts.out = out;
-    BucketSort bs;
+    BucketSort bs{};
     int nb = 0;
     const bool bucket = plan_bucket_sort(T, N, B, L, &bs, &nb);
-    {
-      // a kernel of one block rather than a memset: it starts as the kernel before it ends, and the sort as it ends
-      const int words = kCtlCounts + (bucket ? T * bs.C : 0);
-      SS_TIMED("clear_words_kernel", cs);
-      launch_dependent(clear_words_kernel, 1, words < 1024 ? 128 : 1024, 0, cs, ctl, words);
-    }
+    stt = clear_words(ctl, kCtlCounts + (bucket ? T * bs.C : 0), cs);
+    if (stt != SS_OK) return stt;
     if (bucket) {
       bs.indices = indices; bs.offsets = offsets;
       bs.fallback = ctl + kCtlFallback; bs.ticket = ctl + kCtlTicket; bs.counts = reinterpret_cast<uint32_t*>(ctl + kCtlCounts);
@@ -1767,7 +1758,8 @@ ss_status ss_embbag_bwd_sort_noalloc(int T, int64_t N, const int32_t* indices, c
   ts.keys_a = keys_a; ts.keys_b = keys_b; ts.pos_a = pos_a; ts.pos_b = pos_b; ts.bag_of = bag_of;
   ts.hist = hist; ts.bintot = bintot; ts.tile_heads = heads; ts.ctl = scalars + 8;
   ts.passes = passes; ts.digit_bits = digit_bits; ts.bins = 1 << digit_bits;
-  launch_dependent(clear_words_kernel, 1, 32, 0, cs, ts.ctl, 3);
+  stt = clear_words(ts.ctl, 3, cs);
+  if (stt != SS_OK) return stt;
   const int64_t key_items = ((int64_t)T * B + kSortThreads - 1) / kSortThreads;
   const int64_t tiles = (L + kSortTile - 1) / kSortTile;
   int64_t grid = key_items > tiles ? key_items : tiles;

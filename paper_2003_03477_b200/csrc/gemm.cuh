@@ -12,19 +12,15 @@ namespace ss {
 
 enum OperandKind { OP_F32 = 0, OP_BF16 = 1, OP_F32_ROUND_BF16 = 2 };
 
-struct Epilogue {
+struct Epilogue {               // (no padding: launches are compared byte by byte, see step.cu)
   const float* bias = nullptr;
-  int relu = 0;
   const void* mask = nullptr;   // activation whose sign gates the gradient
-  int mask_bf16 = 0;
   int64_t ld_mask = 0;
-  int mask_cols = 0;
   void* out_lo = nullptr;
-  int lo_bf16 = 0;
   int64_t ld_lo = 0;
-  int lo_cols = 0;
   float* out_hi = nullptr;
   int64_t ld_hi = 0;
+  int relu = 0, mask_bf16 = 0, mask_cols = 0, lo_bf16 = 0, lo_cols = 0, pad = 0;
   // Tensor-core kernels only.  bits_out: besides out_lo (bf16), one bit per element "the stored value is positive",
   // bit n % 32 of word [m * ld_bits_out + n / 32]: the ReLU-gradient mask of the backward pass at 1/16 of the bytes.
   // mask_bits: such a word array of the producing layer; when given it is used instead of `mask` (same meaning).
@@ -46,10 +42,9 @@ struct F32Operand { const float* p; int64_t ld; int k_major, vec; };   // vec: r
 bool f32_operand(const Operand& o, F32Operand* f);                      // false: not float, or neither dimension contiguous
 struct F32Job { int M, N, K, tile0; F32Operand A, B; Epilogue ep; };
 struct F32Jobs {
-  F32Job job[2];
-  int n = 0;
+  F32Job job[2] = {};
   int* clear = nullptr;
-  int clear_words = 0;
+  int n = 0, clear_words = 0;
   bool add(int M, int N, int K, const Operand& A, const Operand& B, const Epilogue& ep) {
     F32Job& J = job[n];
     if (n == 2 || !f32_operand(A, &J.A) || !f32_operand(B, &J.B)) return false;

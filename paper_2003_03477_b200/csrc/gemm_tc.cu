@@ -32,6 +32,7 @@
 // returns; the host reads the flag (ss_device_error).
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <string.h>
 #include <memory>
 #include <mutex>
 #include <vector>
@@ -92,7 +93,7 @@ struct TcParams {
   int dep, dep_mode, dep_k, dep_need;   // see TcJob; dep_need = arrivals that complete a row block of `dep`
   int dep_need_all;        // arrivals that complete all of `dep`
   int signals;             // 1: another product of the flow waits for this one
-  int tma_out;             // 1: outputs leave through shared memory and TMA stores
+  int tma_out, pad;        // tma_out = 1: outputs leave through shared memory and TMA stores
   Epilogue ep;
 };
 
@@ -1087,7 +1088,7 @@ static ss_status flow_plan(const TcJob* jobs, int n, int* ctrl, int max_rows, in
   {
     std::lock_guard<std::mutex> guard(lock);
     for (auto& p : plans)
-      if (p->key == key) { p->used = ++clock; *out = p->flow; return SS_OK; }
+      if (p->key == key) { p->used = ++clock; memcpy(out, &p->flow, sizeof(*out)); return SS_OK; }
   }
   const ss_status st = build_flow(jobs, n, ctrl, max_rows, bn, bn == 256 ? 64 : 128, pair, err, out);
   if (st != SS_OK) return st;
@@ -1100,7 +1101,7 @@ static ss_status flow_plan(const TcJob* jobs, int n, int* ctrl, int max_rows, in
     for (auto& p : plans)                                  // the one not used for longest
       if (!slot || p->used < slot->used) slot = p.get();
   }
-  slot->key = key; slot->flow = *out; slot->used = ++clock;
+  slot->key = key; memcpy(&slot->flow, out, sizeof(*out)); slot->used = ++clock;
   return SS_OK;
 }
 
@@ -1138,7 +1139,13 @@ ss_status gemm_tc_flow(const TcJob* jobs, int n, int* ctrl, int max_rows, int sh
   const bool pair = wide && ctas >= 2 && (ctrl ? t_pair >= 2 * ctas && kb_pair >= 12 * t_pair : t_pair >= ctas / 2);
   const int bn = wide ? 256 : 64;
   alignas(64) TcFlow<kTcMaxFlow> f;
-  const ss_status built = flow_plan(jobs, n, ctrl, max_rows, bn, pair, err, &f);
+  memset(&f, 0, sizeof(f));                                // padding too: launches are compared byte by byte (step.cu)
+  ss_status built;
+  try {
+    built = flow_plan(jobs, n, ctrl, max_rows, bn, pair, err, &f);
+  } catch (...) {                                          // no host memory to keep the block: do without
+    built = build_flow(jobs, n, ctrl, max_rows, bn, bn == 256 ? 64 : 128, pair, err, &f);
+  }
   if (built != SS_OK) return built;
   const int total = f.total_tiles;
   if (pair) {

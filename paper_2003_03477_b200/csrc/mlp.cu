@@ -1,5 +1,6 @@
 // Bottom MLP -> concat -> top MLP -> sigmoid/BCE, its backward pass and the dense Adagrad update.
 #include <cooperative_groups.h>
+#include <string.h>
 #include "gemm.cuh"
 #include "profile.cuh"
 #include "mlp.cuh"
@@ -661,7 +662,7 @@ ss_status mlp_fwd(const ss_mlp_desc* desc, const float* w, const void* w_bf16, c
   cudaStream_t cs = as_stream(stream);
   char* ws = reinterpret_cast<char*>(workspace);
   // the loss kernel's ticket and the control words of the tensor-core flows start at zero (the workspace arrives
-  // uninitialised): the first layer's kernel clears them where it can, else a memset; both clear themselves after use
+  // uninitialised): the first layer's kernel clears them where it can, else clear_words; both clear themselves after use
   int* const ctl = reinterpret_cast<int*>(ws + p.ctrl);
   const int ctl_words = (int)(p.bf16 ? p.ctrl_bytes / 4 : kTicketWords);
   FlowBuilder flow(ctl + kTicketWords, p.ctrl_rows, opt.sharers, cs);
@@ -672,7 +673,7 @@ ss_status mlp_fwd(const ss_mlp_desc* desc, const float* w, const void* w_bf16, c
     const Operand& A = f.A;
     const Operand& Bm = f.Bm;
     const Epilogue& ep = f.ep;
-    if (l == 0 && f.how != FWD_FEW_INPUTS && p.bf16) SS_CUDA(cudaMemsetAsync(ctl, 0, (size_t)ctl_words * 4, cs));
+    if (l == 0 && f.how != FWD_FEW_INPUTS && p.bf16 && (st = clear_words(ctl, ctl_words, cs)) != SS_OK) return st;
     if (l == p.nl - 1) {   // one output unit: a dot product per sample
       st = flow.flush();
       if (st != SS_OK) return st;
@@ -770,7 +771,7 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
 
   float* gpart = reinterpret_cast<float*>(ws + p.gpart);
   GradTable tab;
-  tab.n = 0;
+  memset(&tab, 0, sizeof(tab));                            // unused entries too: launches are compared byte by byte (step.cu)
   auto add_range = [&](int64_t begin, int64_t count, int kind, int64_t off, int64_t stride, int nsplit) {
     const int t = tab.n++;
     tab.begin[t] = begin; tab.end[t] = begin + count; tab.kind[t] = kind; tab.off[t] = off; tab.stride[t] = stride;
@@ -781,7 +782,7 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
   // less for the ordinary model, but sum in another order: one float ulp in a parameter now and then moves its bf16 mirror
   // by an ulp, and the next step's ReLU gates with it.  The update is off the critical path of a step anyway.)
   RedJobs jobs;
-  jobs.njobs = 0; jobs.ntiles = 0; jobs.total = 0;
+  memset(&jobs, 0, sizeof(jobs));
   auto add_job = [&](const void* M, int m_kind, int64_t ldm, int ncols, const void* S, int s_kind, int64_t lds,
                      int s_cols, int64_t out_off) {
     RedJob& J = jobs.job[jobs.njobs++];
@@ -905,7 +906,7 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
   }
   st = flow.flush();
   if (st != SS_OK) return st;
-  if (opt.grads_ready) SS_CUDA(cudaEventRecord(opt.grads_ready, cs));   // grad_pooled is complete
+  if (opt.grads_ready) SS_CUDA(step_record(opt.grads_ready, cs));   // grad_pooled is complete
   float* partial = reinterpret_cast<float*>(ws + p.red_partial);
   if (jobs.njobs > 0) {
     // all batch reductions of the pass in one launch; the update kernel adds the batch slices

@@ -56,6 +56,13 @@ struct Args {
     if (!p && PyErr_Occurred()) throw Bad();
     return static_cast<const ss_mlp_desc*>(p);
   }
+  ss_step_plan plan() {             // None, or the handle as an int
+    PyObject* o = next();
+    if (o == Py_None) return nullptr;
+    void* p = PyLong_AsVoidPtr(o);
+    if (!p && PyErr_Occurred()) throw Bad();
+    return static_cast<ss_step_plan>(p);
+  }
   // None: torch's current stream; an object with .cuda_stream; or the handle as an int
   ss_stream stream() {
     PyObject* o = next();
@@ -284,6 +291,7 @@ SS_PY(train_step) {
     s.lr = a.f32(); s.eps = a.f32();
     s.replicas = a.i32();
     s.stream = a.stream(); s.sort_stream = a.stream(); s.mlp_stream = a.stream();
+    s.plan = a.plan();
     NoGil released;
     return ss_train_step(&s);
   });

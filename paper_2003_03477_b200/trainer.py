@@ -104,6 +104,7 @@ class Replica:
         # so it goes in between where the device has a level left (measured +2 % examples/s)
         self.side = torch.cuda.Stream(device=dev, priority=model.prio_sort)
         self.mlp = torch.cuda.Stream(device=dev, priority=priority)
+        self.plan = ss.StepPlan()                  # the step as a graph, once it has been taken often enough
         self.steps_done = 0
 
 
@@ -170,7 +171,7 @@ class Model:
                          batch.L, batch.dense, batch.labels, rep.w, rep.w_bf16, rep.acc, rep.concat_f32, rep.concat_bf16,
                          rep.logit, rep.prob, rep.loss, rep.grad_pooled, rep.mlp_ws, rep.emb_ws, rep.uniq_keys, rep.seg_off,
                          rep.perm, rep.num_unique, self.d_status, self.lr, self.eps, self.sharers, s, rep.side if overlap_sort else s,
-                         rep.mlp if s is rep.stream else s)
+                         rep.mlp if s is rep.stream else s, rep.plan)
         rep.steps_done += 1
 
     # ---------------------------------------------------------------- one synchronisation pass

@@ -80,3 +80,10 @@ def test_binding_constants_match_the_header():
     hdr = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "include", "shadowsync.h")).read()
     m = re.search(r"#define\s+SS_TABLE_SORT_CAP\s+(\d+)", hdr)
     assert m and int(m.group(1)) == ss.SS_TABLE_SORT_CAP
+
+
+def test_step_plans_need_no_device(lib):
+    """A plan starts empty, is freed with its object, and NULL is refused or ignored."""
+    assert ss.StepPlan().counts() == (0, 0, 0, 0)
+    assert lib.ss_step_plan_create(None) == -1 and lib.ss_step_plan_counts(None, (C.c_int64 * 4)()) == -1
+    lib.ss_step_plan_destroy(None)
