@@ -135,7 +135,7 @@ struct BwdPlan {
   int nwin;
   size_t off_keys_a, off_keys_b, off_pos_a, off_pos_b, off_bag, off_hist, off_bintot, off_heads, off_uniq, off_seg,
       off_uidx, off_sbag, off_partial, off_long, off_gsum, off_scalars, off_ctl, total;
-  size_t ctl_bytes;  // control words of the sort kernels, cleared by one memset: see kCtlFallback ...
+  size_t ctl_bytes;  // control words of the sort kernels, cleared before them: see kCtlFallback ...
 };
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -606,20 +606,26 @@ tiled_sort_kernel(const __grid_constant__ TiledSort a) {
 
 // ---- (2b) bucket sort in shared memory ------------------------------------------------------------
 // The lookups arrive grouped by table (bags are table-major), so the sort by key = t*N + row is T independent sorts by
-// row.  A table is cut into C ranges of rows and a block takes one range: it reads the table's whole index list (C times
-// L2 traffic, a few bytes per lookup), keeps the lookups of its range in order, and sorts them in shared memory with
+// row.  A table is cut into ranges of rows and a block takes one range: it reads the table's whole index list (a few bytes
+// of L2 traffic per lookup), keeps the lookups of its range in order, and sorts them in shared memory with
 // stable LSD passes over the bits of the range alone.  Ranges share no row, so the block also finds its distinct rows by
-// itself; only the number of distinct rows before it comes from the other blocks (a published count per block, summed by
+// itself; only the number of distinct rows before it comes from the other blocks (a published count per range, summed by
 // everybody), and all outputs of the sort half leave from here: one launch instead of sort, count, scan and write.
-// Blocks take their range from a ticket, so the counts a block waits for come from blocks that are running.
-// What bounds it is instruction issue and the latency of a block's rounds.  Measured alone: 26 tables of 21 500 lookups
-// 47 us (53 us for a sort with one block per table, and 25 us for the count, scan and write launches behind it), 26 tables
-// of 33 400 lookups 52 us (tiled passes 127 us), 40 tables of 33 500 lookups 58 us on 120 blocks (tiled passes 200 us).
+// Blocks take their ranges from a ticket, so the counts a block waits for come from blocks that are running.  There are as
+// many blocks as tables of any lengths could need; those without a range leave at once.
 //
-// A block that cannot take the path (more than `cap` lookups in its range, a table of more than 65536, offsets that are
-// not monotone within [0, L], a row index outside the table) raises *fallback.  Only a range can be too full if L > cap:
-// then the caller launches tiled_sort_kernel behind this kernel, which returns at once when the flag is down.  Otherwise
-// the input is malformed, and the last block to leave runs the tiled sort's items by itself: slow, and nothing to launch.
+// The cut follows the data.  A table gets a range per `per_range` of its own lookups, and the ranges hold about equally
+// many: their edges are quantiles of 2048 lookups spread over the table, which every block of the table reads alike.  So it
+// does not matter whether popular rows are scattered or neighbours, or one table is longer than another.  A popular row on
+// an edge goes to the side that has less of it; where a range is too full all the same, because its first or last row draws
+// so much, that row is not sorted but copied out, in order, by a second walk over the index list.
+// What bounds it is instruction issue and the latency of a block's rounds.
+//
+// A block that cannot take the path (a range with more lookups than `cap` after all, a table of more than 65536, offsets
+// that are not monotone within [0, L], a row index outside the table) raises *fallback.  Only a range can be too full if
+// L > cap: then the caller launches tiled_sort_kernel behind this kernel, which returns at once when the flag is down.
+// Otherwise the input is malformed, and the last block to leave runs the tiled sort's items by itself: slow, and nothing
+// to launch.
 constexpr int kBsThreads = 1024;
 constexpr int kBsWarps = kBsThreads / 32;
 constexpr int kBsChunk = 8 * kBsThreads;                   // index positions looked at together, 8 per thread
@@ -627,6 +633,9 @@ constexpr int kBsDigit = 10;                               // most bits of a dig
 constexpr int kBsMaxLookups = 65536;                       // of a table: positions inside it take 16 bits
 constexpr size_t kBsSmemMax = 226 * 1024;                  // leaves room for the static part
 constexpr int kBsRounds = 16;                              // most rounds of 32 lookups per warp: a block sorts up to 16384
+// Lookups a range is meant to hold: with kBsSamples the share of a range of C equal ones is off by sqrt((C - 1) / 2048) of
+// itself (one standard deviation), so 13400 stays below 16384 by five of them for up to five ranges.
+constexpr int kBsSamples = 2 * kBsThreads, kBsRange = 13400;
 // dynamic shared memory: row, position, bag and index of the kept lookups (10 bytes each), then a region that first
 // holds a chunk of the index list and its bags and later the digit counters
 __host__ __device__ constexpr size_t bs_counter_bytes(int nb) { return (size_t)kBsWarps * ((1 << nb) + 2) * 2; }
@@ -637,19 +646,18 @@ __host__ __device__ constexpr size_t bs_smem(int cap, int nb) {
   const size_t own = (size_t)cap * 10 + bs_region(nb), tiled = sort_smem_words(kBsThreads) * 4;
   return own > tiled ? own : tiled;
 }
-constexpr int bs_cap(int nb) {
-  const int room = (int)((kBsSmemMax - bs_region(nb)) / 10) & ~31;
-  return room < kBsRounds * kBsThreads ? room : kBsRounds * kBsThreads;
-}
+constexpr int kBsCap = kBsRounds * kBsThreads;
+static_assert(bs_smem(kBsCap, kBsDigit) <= kBsSmemMax, "the largest range and the widest digit fit");
 
 struct BucketSort {
   const int32_t* indices; const int32_t* offsets;
-  int T, B; int64_t N;
-  int C, rows_per, cap, passes;                            // buckets per table, rows of one, lookups one can hold, digit passes
+  int64_t N;
+  int T, B;
+  int per_range, cap;                                      // lookups per range, lookups one can hold
+  int ranges, serial_fallback;                             // ranges > 0: that many for every table (more tables than threads)
   int32_t* fallback;                                       // zero at launch
-  int* ticket;                                             // {next block, blocks gone}: zero at launch
-  uint32_t* counts;                                        // [T * C], zero at launch: distinct rows of a block | 1 << 31
-  int serial_fallback;
+  int* ticket;                                             // {next range, blocks gone}: zero at launch
+  uint32_t* counts;                                        // [T * kBsMaxBuckets], zero at launch: distinct rows of a range | 1 << 31
 };
 
 template <int NB>
@@ -664,52 +672,134 @@ __device__ __forceinline__ uint32_t same_digit_lanes_n(uint32_t digit) {
   return peers;
 }
 
-template <int NB>                                          // digit bits, 5..kBsDigit
-__global__ void __launch_bounds__(kBsThreads, 1)
-bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__ TiledSort tiled) {
-  wait_for_previous_kernel();
-  extern __shared__ __align__(16) unsigned char bs_raw[];
+// One stable LSD pass over NB bits of the kept lookups' rows: order -> order.  A pass looks at every lookup once: the lanes
+// of a round that hold the same digit give its rank among the warp's lookups with that digit, kept in a register until the
+// counters have been scanned.
+template <int NB>
+__device__ __forceinline__ void bucket_sort_pass(const uint32_t* okey, uint16_t* order, uint16_t* cnt, uint32_t* s_w, int shift,
+                                                 int i0, int iend) {
   constexpr int bins = 1 << NB, kStride = bins + 2;        // padded: the scan reads one digit of all warps
   constexpr uint32_t mask = (uint32_t)bins - 1u;
-  const SortOut& o = tiled.out;
-  const int cap = a.cap;
-  uint32_t* okey = reinterpret_cast<uint32_t*>(bs_raw);    // row, relative to the range, of kept lookup i
-  uint16_t* opos = reinterpret_cast<uint16_t*>(okey + cap);           // its position in the table
-  uint16_t* obag = opos + cap;                             // its bag, inside the table
-  uint16_t* order = obag + cap;                            // the kept lookups in the order reached so far
-  uint16_t* cnt = order + cap;                             // [kBsWarps][kStride]
-  uint32_t* crow = reinterpret_cast<uint32_t*>(cnt);       // the chunk's row ids (cap is a multiple of 32: 16-byte aligned)
-  uint16_t* cbag = reinterpret_cast<uint16_t*>(crow + kBsChunk);      // and bags
-  __shared__ uint32_t s_w[kBsWarps], s_m[kBsWarps];
-  __shared__ uint32_t s_scalar[4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_scalar[0] = (uint32_t)atomicAdd(a.ticket, 1);
+  uint16_t* mycnt = cnt + warp * kStride;
+  uint32_t held[kBsRounds];                                // lookup | rank << 16
+  for (int i = tid; i < kBsWarps * kStride / 2; i += kBsThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
   __syncthreads();
-  const int id = (int)s_scalar[0];
-  const int t = id / a.C, c = id - t * a.C;
-  const int64_t bag0 = (int64_t)t * a.B;
-  const int seg0 = a.offsets[bag0], seg1 = a.offsets[bag0 + a.B];
-  const uint32_t lo = (uint32_t)c * (uint32_t)a.rows_per;
-  const uint32_t span = c == a.C - 1 ? (uint32_t)a.N - lo : (uint32_t)a.rows_per;
-  // block-uniform checks of the table's segment
-  bool ok = seg0 >= 0 && seg1 >= seg0 && (int64_t)seg1 <= o.L && seg1 - seg0 <= kBsMaxLookups && (t != 0 || seg0 == 0) &&
-            (t != a.T - 1 || (int64_t)seg1 == o.L);
-  const int n = ok ? seg1 - seg0 : 0;
-  int kept = 0;                                            // lookups of the range so far
-  int below = 0;                                           // per thread: lookups of smaller ranges
-  // the index list goes through shared memory so that its loads are coalesced; a chunk's loads are in flight while the
-  // chunk before is worked on, and the first bags' offsets while the first chunk arrives
-  uint32_t next[8];
-  auto request = [&](int p0) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int p = p0 + tid + k * kBsThreads;
-      next[k] = p < n ? (uint32_t)__ldg(a.indices + seg0 + p) : 0u;
+  for (int r = 0; r < kBsRounds; ++r) {                    // whole rounds: the bounds are the same for all lanes
+    const int i = i0 + 32 * r + lane;
+    if (i - lane >= iend) break;
+    const uint32_t pay = shift == 0 ? (uint32_t)i : order[i];
+    const uint32_t digit = (okey[pay] >> shift) & mask;
+    const uint32_t peers = same_digit_lanes_n<NB>(digit);
+    const uint32_t lower = peers & ((1u << lane) - 1u);
+    const uint32_t base = mycnt[digit];
+    __syncwarp();
+    if (lower == 0) mycnt[digit] = (uint16_t)(base + __popc(peers));
+    __syncwarp();
+    held[r] = pay | (base + __popc(lower)) << 16;
+  }
+  __syncthreads();
+  // exclusive scan in (digit, warp) order: thread tid owns bins / 32 consecutive entries of that order
+  {
+    constexpr int per = bins >> 5;
+    uint32_t v[per], sum = 0;
+#pragma unroll
+    for (int u = 0; u < per; ++u) {
+      const int e = tid * per + u;
+      v[u] = cnt[(e & 31) * kStride + (e >> 5)];
+      sum += v[u];
     }
-  };
-  request(0);
-  int first_l = 0, first_h = 0;                            // offsets of bag `tid`
-  if (tid < a.B) { first_l = a.offsets[bag0 + tid]; first_h = a.offsets[bag0 + tid + 1]; }
+    uint32_t run = block_scan<kBsThreads>(sum, s_w) - sum;
+#pragma unroll
+    for (int u = 0; u < per; ++u) {
+      const int e = tid * per + u;
+      cnt[(e & 31) * kStride + (e >> 5)] = (uint16_t)run;
+      run += v[u];
+    }
+  }
+  __syncthreads();
+  // stable scatter
+#pragma unroll
+  for (int r = 0; r < kBsRounds; ++r) {
+    if (i0 + 32 * r >= iend) break;
+    const uint32_t pay = held[r] & 0xffffu;
+    order[mycnt[(okey[pay] >> shift) & mask] + (held[r] >> 16)] = (uint16_t)pay;
+  }
+  __syncthreads();
+}
+
+// The range in hand: what one phase finds out and a later one needs stays in shared memory rather than in registers.
+struct BucketRange {
+  uint32_t w[kBsWarps], m[kBsWarps];                       // scratch of the scans
+  uint32_t total, id;                                      // ranges of all tables, this one
+  int t, c, ranges, seg0, seg1;                            // its table, its number there, how many there are, the table's segment
+  uint32_t edge[2], rank[2];                               // while the edges are looked for
+  uint32_t base, span, hot_row;                            // rows [base, base + span) are sorted, one beside them may be copied out
+  int kept, hot, out0;                                     // lookups sorted and copied out, where the sorted ones go
+  uint32_t mine, before;                                   // distinct rows of this range and of those before it
+};
+
+__device__ __forceinline__ bool sound_table(const BucketSort& a, int64_t L, int t, int seg0, int seg1) {
+  return seg0 >= 0 && seg1 >= seg0 && (int64_t)seg1 <= L && seg1 - seg0 <= kBsMaxLookups && (t != 0 || seg0 == 0) &&
+         (t != a.T - 1 || (int64_t)seg1 == L);
+}
+
+// Two edges of a table's ranges, into r.edge: the k0-th and k1-th smallest (from 0) of the threads' 2 x 1024 values, below
+// 2^bits, each plus one if more of the values equal to it come before that place than after.  A histogram of the highest ten
+// bits tells in which bin each lies, one of the next ten bits of that bin's values the bin inside it, and so on.  Counts of
+// the two share a word.  hist: 1024 words of shared memory.
+__device__ __forceinline__ void select_two(BucketRange& r, uint32_t* hist, const uint32_t (&value)[2], int bits, int k0, int k1) {
+  const int tid = threadIdx.x;
+  if (tid == 0) { r.edge[0] = r.edge[1] = 0u; r.rank[0] = (uint32_t)k0; r.rank[1] = (uint32_t)k1; }
+  for (int shift = bits; shift > 0;) {
+    const int d = shift < 10 ? shift : 10;
+    shift -= d;
+    hist[tid] = 0u;
+    __syncthreads();
+    const uint32_t e0 = r.edge[0], e1 = r.edge[1], want0 = r.rank[0], want1 = r.rank[1];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const uint32_t high = value[i] >> shift >> d, add = (high == e0 ? 1u : 0u) + (high == e1 ? 0x10000u : 0u);
+      if (add) atomicAdd(&hist[(value[i] >> shift) & ((1u << d) - 1u)], add);
+    }
+    __syncthreads();
+    const uint32_t own = hist[tid];                        // (bins beyond 2^d are empty)
+    const uint32_t upto = block_scan<kBsThreads>(own, r.w), before = upto - own;
+    const uint32_t at0 = want0 - (before & 0xffffu), at1 = want1 - (before >> 16);
+    if (at0 < (own & 0xffffu)) { r.edge[0] = (e0 << d | (uint32_t)tid) + (shift == 0 && 2 * at0 > (own & 0xffffu)); r.rank[0] = at0; }
+    if (at1 < own >> 16) { r.edge[1] = (e1 << d | (uint32_t)tid) + (shift == 0 && 2 * at1 > own >> 16); r.rank[1] = at1; }
+    __syncthreads();
+  }
+}
+
+constexpr uint32_t kNoRow = 0xffffffffu;                   // no row id is that large
+// What a thread has in flight before a walk: the first chunk of the index list, the offsets of bag `tid`.
+struct WalkStart {
+  uint32_t next[8];
+  int l, h;
+  __device__ __forceinline__ WalkStart(const BucketSort& a, const BucketRange& r, int n) {
+    const int tid = threadIdx.x;
+    const int32_t* off = a.offsets + (int64_t)r.t * a.B;
+    l = h = 0;
+    if (tid < a.B) { l = off[tid]; h = off[tid + 1]; }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) next[k] = tid + k * kBsThreads < n ? (uint32_t)__ldg(a.indices + r.seg0 + tid + k * kBsThreads) : 0u;
+  }
+};
+
+// Walks the index list of table r.t, n long, and hands the lookups of rows [from, from + rows) to put(number, number in the
+// chunk, row, position, bag), in order, and after each chunk their numbers to flush(first, count); their count, or -1: more
+// than `limit`, or malformed.  Per thread, `seen` counts the lookups of rows before `from`, and in its upper half those of
+// row `hot`.  The list goes through shared memory so that its loads are coalesced; a chunk's loads are in flight while the
+// chunk before is worked on.
+template <typename Put, typename Flush>
+__device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, uint32_t* crow, uint16_t* cbag, int n, WalkStart& start,
+                                          uint32_t from, uint32_t rows, uint32_t hot, int limit, uint32_t& seen, Put put, Flush flush) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int seg0 = r.seg0, seg1 = seg0 + n;
+  const int32_t* off = a.offsets + (int64_t)r.t * a.B;
+  int kept = 0;
   uint32_t bag_carry = 0;                                  // 1 + the last bag that starts before the chunk
   for (int p0 = 0; p0 == 0 || p0 < n; p0 += kBsChunk) {    // (once for an empty table: its offsets are checked here)
     const int p1 = min(n, p0 + kBsChunk);
@@ -723,12 +813,16 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
     };
     *reinterpret_cast<uint4*>(cbag + 8 * tid) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    if (tid < a.B) mark(tid, first_l, first_h);
+    if (tid < a.B) mark(tid, start.l, start.h);
 #pragma unroll 2
-    for (int b = tid + kBsThreads; b < a.B; b += kBsThreads) mark(b, a.offsets[bag0 + b], a.offsets[bag0 + b + 1]);
+    for (int b = tid + kBsThreads; b < a.B; b += kBsThreads) mark(b, off[b], off[b + 1]);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) crow[tid + k * kBsThreads] = next[k];
-    request(p0 + kBsChunk);
+    for (int k = 0; k < 8; ++k) crow[tid + k * kBsThreads] = start.next[k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int p = p0 + kBsChunk + tid + k * kBsThreads;
+      start.next[k] = p < n ? (uint32_t)__ldg(a.indices + seg0 + p) : 0u;
+    }
     __syncthreads();
     const uint4 r0 = *reinterpret_cast<const uint4*>(crow + 8 * tid), r1 = *reinterpret_cast<const uint4*>(crow + 8 * tid + 4);
     const uint32_t row[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
@@ -737,10 +831,14 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
     for (int k = 0; k < 8; ++k) {
       const bool in = w0 + k < p1;
       if (in && row[k] >= (uint32_t)a.N) bad = 1;          // one unsigned compare: negative indices are huge
-      mine += in && row[k] - lo < span;
-      below += in && row[k] < lo;
+      mine += in && row[k] - from < rows;
+      seen += in && row[k] < from;
     }
-    if (__syncthreads_or(bad)) { ok = false; break; }
+    if (hot != kNoRow) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) seen += w0 + k < p1 && row[k] == hot ? 0x10000u : 0u;   // at most 64 positions a thread
+    }
+    if (__syncthreads_or(bad)) return -1;
     const uint4 mk = *reinterpret_cast<const uint4*>(cbag + 8 * tid);
     const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
     uint32_t top = 0;                                      // the highest number at this thread's positions
@@ -749,21 +847,21 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
     // scan over the threads: kept lookups (sum) and bag numbers (maximum)
     uint32_t sum = (uint32_t)mine, mx = top;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t u = __shfl_up_sync(0xffffffffu, sum, off), v = __shfl_up_sync(0xffffffffu, mx, off);
-      if (lane >= off) { sum += u; mx = max(mx, v); }
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, sum, d), v = __shfl_up_sync(0xffffffffu, mx, d);
+      if (lane >= d) { sum += u; mx = max(mx, v); }
     }
-    if (lane == 31) { s_w[warp] = sum; s_m[warp] = mx; }
+    if (lane == 31) { r.w[warp] = sum; r.m[warp] = mx; }
     __syncthreads();
-    uint32_t ws = s_w[lane], wm = s_m[lane];               // kBsWarps == 32: every warp scans the warps' totals
+    uint32_t ws = r.w[lane], wm = r.m[lane];               // kBsWarps == 32: every warp scans the warps' totals
     const uint32_t ws0 = ws;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t u = __shfl_up_sync(0xffffffffu, ws, off), v = __shfl_up_sync(0xffffffffu, wm, off);
-      if (lane >= off) { ws += u; wm = max(wm, v); }
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, ws, d), v = __shfl_up_sync(0xffffffffu, wm, d);
+      if (lane >= d) { ws += u; wm = max(wm, v); }
     }
     const int chunk = (int)__shfl_sync(0xffffffffu, ws, 31);
-    if (kept + chunk > cap) { ok = false; break; }         // the range is too full
+    if (kept + chunk > limit) return -1;
     int at = kept + (int)(__shfl_sync(0xffffffffu, ws - ws0, warp) + sum) - mine;
     uint32_t bag = __shfl_up_sync(0xffffffffu, mx, 1);
     if (lane == 0) bag = 0;
@@ -773,152 +871,212 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       bag = max(bag, (k & 1) ? mw[k >> 1] >> 16 : mw[k >> 1] & 0xffffu);
-      if (w0 + k < p1 && row[k] - lo < span) {
-        okey[at] = row[k] - lo;
-        opos[at] = (uint16_t)(w0 + k);
-        obag[at] = (uint16_t)(bag - 1);
+      if (w0 + k < p1 && row[k] - from < rows) {
+        put(at, at - kept, row[k], w0 + k, (int)bag - 1);
         ++at;
       }
     }
+    __syncthreads();                                       // the chunk's bags and the scans' scratch are free again
+    flush(kept, chunk);
     kept += chunk;
-    __syncthreads();                                       // the chunk's bags and s_w are free again
   }
-  const int q = ok ? kept : 0, q32 = (q + 31) & ~31;
-  if (!ok && tid == 0) atomicOr(a.fallback, 1);
-  // pads of the last round: the largest digits and the last places, so every stable pass leaves them at the end
-  __syncthreads();
-  if (tid < q32 - q) okey[q + tid] = 0xffffffffu;
-  // where the range starts in the sorted order
-  for (int off = 16; off >= 1; off >>= 1) below += __shfl_down_sync(0xffffffffu, below, off);
-  if (lane == 0) s_w[warp] = (uint32_t)below;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t v = s_w[lane];
-    for (int off = 16; off >= 1; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) s_scalar[1] = v;
-  }
-  __syncthreads();
-  const int out0 = seg0 + (int)s_scalar[1];
-  const int rounds = (q32 + kBsThreads - 1) / kBsThreads;  // rounds of 32 consecutive items per warp
-  const int i0 = warp * rounds * 32, iend = min(i0 + rounds * 32, q32);
-  uint16_t* mycnt = cnt + warp * kStride;
-  // A pass looks at every lookup once: the lanes of a round that hold the same digit give its rank among the warp's
-  // lookups with that digit, kept in a register until the counters have been scanned.
-  uint32_t held[kBsRounds];                                // lookup | rank << 16
-  for (int pass = 0; pass < (q > 0 ? a.passes : 0); ++pass) {
-    const int shift = pass * NB;
-    for (int i = tid; i < kBsWarps * kStride / 2; i += kBsThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0u;
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kBsRounds; ++r) {                  // whole rounds: the bounds are the same for all lanes
-      const int i = i0 + 32 * r + lane;
-      if (i - lane >= iend) break;
-      const uint32_t pay = pass == 0 ? (uint32_t)i : order[i];
-      const uint32_t digit = (okey[pay] >> shift) & mask;
-      const uint32_t peers = same_digit_lanes_n<NB>(digit);
-      const uint32_t lower = peers & ((1u << lane) - 1u);
-      const uint32_t base = mycnt[digit];
-      __syncwarp();
-      if (lower == 0) mycnt[digit] = (uint16_t)(base + __popc(peers));
-      __syncwarp();
-      held[r] = pay | (base + __popc(lower)) << 16;
+  return kept;
+}
+
+template <int NB>                                          // digit bits, 5..kBsDigit
+__global__ void __launch_bounds__(kBsThreads, 1)
+bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__ TiledSort tiled) {
+  wait_for_previous_kernel();
+  extern __shared__ __align__(16) unsigned char bs_raw[];
+  __shared__ BucketRange r;
+  const SortOut& o = tiled.out;
+  const int cap = a.cap;
+  uint32_t* okey = reinterpret_cast<uint32_t*>(bs_raw);    // row, relative to the range, of kept lookup i
+  uint16_t* opos = reinterpret_cast<uint16_t*>(okey + cap);           // its position in the table
+  uint16_t* obag = opos + cap;                             // its bag, inside the table
+  uint16_t* order = obag + cap;                            // the kept lookups in the order reached so far
+  uint16_t* cnt = order + cap;                             // [kBsWarps][bins + 2]
+  uint32_t* crow = reinterpret_cast<uint32_t*>(cnt);       // the chunk's row ids (cap is a multiple of 32: 16-byte aligned)
+  uint16_t* cbag = reinterpret_cast<uint16_t*>(crow + kBsChunk);      // and bags
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  do {                                                     // (a break: nothing to do for this block)
+    // ---- how many ranges every table has, by its lookups, and which range is this block's; thread t looks after table t
+    if (a.ranges == 0) {
+      constexpr int kBad = 1 << 20;                        // more than all ranges
+      int first = 0, last = 0, mine = 0;
+      if (tid < a.T) {
+        first = a.offsets[(int64_t)tid * a.B];
+        last = a.offsets[(int64_t)(tid + 1) * a.B];
+      }
+      if (tid == 0) r.id = (uint32_t)atomicAdd(a.ticket, 1);
+      if (tid < a.T)
+        mine = sound_table(a, o.L, tid, first, last) ? max(1, min(kBsMaxBuckets, (last - first + a.per_range - 1) / a.per_range)) : kBad;
+      const int end = (int)block_scan<kBsThreads>((uint32_t)mine, r.w), id = (int)r.id;
+      if (tid == kBsThreads - 1) {
+        r.total = (uint32_t)end;
+        if (end >= kBad) atomicOr(a.fallback, 1);
+      }
+      if (id < end && id >= end - mine) { r.t = tid; r.c = id - (end - mine); r.ranges = mine; r.seg0 = first; r.seg1 = last; }
+      __syncthreads();
+      if (r.id >= r.total || r.total >= (uint32_t)kBad) break;
+    } else {
+      if (tid == 0) {
+        r.id = (uint32_t)atomicAdd(a.ticket, 1);
+        const int t = (int)r.id / a.ranges;
+        r.total = gridDim.x;
+        r.t = t; r.c = (int)r.id - t * a.ranges; r.ranges = a.ranges;
+        r.seg0 = a.offsets[(int64_t)t * a.B]; r.seg1 = a.offsets[(int64_t)(t + 1) * a.B];
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    // exclusive scan in (digit, warp) order: thread tid owns bins / 32 consecutive entries of that order
+    // ---- the range's rows, and its lookups into shared memory
     {
-      constexpr int per = bins >> 5;
-      uint32_t v[per], sum = 0;
+      const bool sound = sound_table(a, o.L, r.t, r.seg0, r.seg1);
+      const int n = sound ? r.seg1 - r.seg0 : 0, C = r.ranges;
+      uint32_t sample[2] = {0u, 0u};
+      if (C > 1 && n > 0) {
 #pragma unroll
-      for (int u = 0; u < per; ++u) {
-        const int e = tid * per + u;
-        v[u] = cnt[(e & 31) * kStride + (e >> 5)];
-        sum += v[u];
+        for (int i = 0; i < 2; ++i)
+          sample[i] = min((uint32_t)__ldg(a.indices + r.seg0 + (((2 * tid + i) * n) >> 11)), (uint32_t)a.N - 1u);
       }
-      uint32_t run = block_scan<kBsThreads>(sum, s_w) - sum;
-#pragma unroll
-      for (int u = 0; u < per; ++u) {
-        const int e = tid * per + u;
-        cnt[(e & 31) * kStride + (e >> 5)] = (uint16_t)run;
-        run += v[u];
+      WalkStart start(a, r, n);
+      uint32_t lo = 0, hi = (uint32_t)a.N, hot = kNoRow;   // hot: the row that is copied out
+      if (C > 1 && n > 0) {
+        const int c = r.c, bits = max(1, 32 - __clz((uint32_t)a.N - 1u));
+        select_two(r, okey, sample, bits, c * kBsSamples / C, min((c + 1) * kBsSamples / C, kBsSamples - 1));
+        if (c > 0) lo = r.edge[0];
+        if (c < C - 1) hi = r.edge[1];
+        auto count = [&](uint32_t from, uint32_t rows) {   // samples of rows [from, from + rows)
+          return __syncthreads_count(sample[0] - from < rows) + __syncthreads_count(sample[1] - from < rows);
+        };
+        // five standard deviations of the samples' share below what the block can hold (1 / 18 = 2.5 / sqrt(2048))
+        if ((int64_t)count(lo, hi - lo) * n > (int64_t)(cap - n / 18) * kBsSamples) hot = count(lo, 1u) >= count(hi - 1u, 1u) ? lo : hi - 1u;
       }
+      const uint32_t base = lo + (hot == lo), span = hi - base - (hot != lo && hot != kNoRow);
+      uint32_t seen = 0;
+      const int kept = walk_table(a, r, crow, cbag, n, start, base, span, hot, cap, seen,
+                                  [&](int at, int, uint32_t row, int position, int bag) {
+                                    okey[at] = row - base;
+                                    opos[at] = (uint16_t)position;
+                                    obag[at] = (uint16_t)bag;
+                                  }, [](int, int) {});
+      const bool ok = sound && kept >= 0;
+      if (!ok && tid == 0) atomicOr(a.fallback, 1);
+      const int q = ok ? kept : 0;
+      // pads of the last round: the largest digits and the last places, so every stable pass leaves them at the end
+      __syncthreads();
+      if (tid < ((q + 31) & ~31) - q) okey[q + tid] = 0xffffffffu;
+      const uint32_t below = __reduce_add_sync(0xffffffffu, seen & 0xffffu), n_hot = __reduce_add_sync(0xffffffffu, seen >> 16);
+      if (lane == 0) { r.w[warp] = below; r.m[warp] = n_hot; }
+      __syncthreads();
+      if (warp == 0) {
+        const int all_below = (int)__reduce_add_sync(0xffffffffu, r.w[lane]), all_hot = (int)__reduce_add_sync(0xffffffffu, r.m[lane]);
+        if (lane == 0) {
+          r.base = base; r.span = span; r.hot_row = hot; r.kept = q;
+          r.hot = ok ? all_hot : 0;
+          r.out0 = r.seg0 + all_below;
+        }
+      }
+      __syncthreads();
+    }
+    // ---- sort
+    const int q = r.kept, q32 = (q + 31) & ~31;
+    const int rounds = (q32 + kBsThreads - 1) / kBsThreads;  // rounds of 32 consecutive items per warp
+    const int i0 = warp * rounds * 32, iend = min(i0 + rounds * 32, q32);
+    if (q > 0) {
+      const int bits = max(1, 32 - __clz(r.span - 1u));    // (something was kept: there is a row)
+      for (int shift = 0; shift < bits; shift += NB) bucket_sort_pass<NB>(okey, order, cnt, r.w, shift, i0, iend);
+    }
+    // ---- distinct rows: a warp walks its sorted positions 32 at a time; a position is a head when its row differs from the one before
+    auto head_at = [&](int j, uint32_t k) {                // all lanes; k: row at j (anything beyond the end)
+      uint32_t before = __shfl_up_sync(0xffffffffu, k, 1);
+      if (lane == 0) before = j > 0 && j <= q ? okey[order[j - 1]] : 0u;
+      return j < q && (j == 0 || k != before);
+    };
+    uint32_t heads = 0;
+    for (int j = i0 + lane; j < iend; j += 32) heads += __popc(__ballot_sync(0xffffffffu, head_at(j, okey[order[j]])));
+    const uint32_t inc = block_scan<kBsThreads>(lane == 0 ? heads : 0u, r.w);   // heads of the warps up to this one
+    if (tid == kBsThreads - 1) {
+      r.mine = inc + (r.hot > 0);
+      atomicExch(a.counts + r.id, r.mine | 0x80000000u);   // for the ranges behind this one
     }
     __syncthreads();
-    // stable scatter
-#pragma unroll
-    for (int r = 0; r < kBsRounds; ++r) {
-      if (i0 + 32 * r >= iend) break;
-      const uint32_t pay = held[r] & 0xffffu;
-      order[mycnt[(okey[pay] >> shift) & mask] + (held[r] >> 16)] = (uint16_t)pay;
+    // distinct rows of the ranges before this one
+    {
+      uint32_t sum = 0;
+      bool gave_up = false;
+      const long long t0 = clock64();
+      for (int i = tid; i < (int)r.id; i += kBsThreads) {
+        uint32_t v;
+        while (!((v = *reinterpret_cast<volatile uint32_t*>(a.counts + i)) >> 31)) {
+          if (clock64() - t0 > 2000000000ll) { gave_up = true; break; }
+          __nanosleep(64);
+        }
+        sum += v & 0x7fffffffu;
+      }
+      if (gave_up && o.d_status) atomicOr(o.d_status, SS_DEV_BAD_WORKSPACE);
+      const uint32_t all = block_scan<kBsThreads>(sum, r.w);
+      if (tid == kBsThreads - 1) r.before = all;
     }
     __syncthreads();
-  }
-  // distinct rows: a warp walks its sorted positions 32 at a time; a position is a head when its row differs from the one before
-  auto head_at = [&](int j, uint32_t k) {                  // all lanes; k: row at j (anything beyond the end)
-    uint32_t before = __shfl_up_sync(0xffffffffu, k, 1);
-    if (lane == 0) before = j > 0 && j <= q ? okey[order[j - 1]] : 0u;
-    return j < q && (j == 0 || k != before);
-  };
-  uint32_t heads = 0;
-  for (int j = i0 + lane; j < iend; j += 32) heads += __popc(__ballot_sync(0xffffffffu, head_at(j, okey[order[j]])));
-  const uint32_t inc = block_scan<kBsThreads>(lane == 0 ? heads : 0u, s_w);   // heads of the warps up to this one
-  if (tid == kBsThreads - 1) {
-    s_scalar[2] = inc;
-    atomicExch(a.counts + id, inc | 0x80000000u);          // for the blocks behind this one
-  }
-  __syncthreads();
-  // distinct rows of the blocks before this one
-  {
-    uint32_t sum = 0;
-    bool gave_up = false;
-    const long long t0 = clock64();
-    for (int i = tid; i < id; i += kBsThreads) {
-      uint32_t v;
-      while (!((v = *reinterpret_cast<volatile uint32_t*>(a.counts + i)) >> 31)) {
-        if (clock64() - t0 > 2000000000ll) { gave_up = true; break; }
-        __nanosleep(64);
-      }
-      sum += v & 0x7fffffffu;
-    }
-    if (gave_up && o.d_status) atomicOr(o.d_status, SS_DEV_BAD_WORKSPACE);
-    const uint32_t all = block_scan<kBsThreads>(sum, s_w);
-    if (tid == kBsThreads - 1) s_scalar[3] = all;
-  }
-  __syncthreads();
-  const uint32_t u0 = s_scalar[3], mine_u = s_scalar[2];
-  // outputs
-  const uint32_t key0 = (uint32_t)((uint64_t)t * (uint64_t)a.N) + lo;
-  uint32_t u_next = u0 + __shfl_sync(0xffffffffu, inc - (lane == 0 ? heads : 0u), 0);
+    // ---- outputs: the sorted rows, and the row copied out before or behind them
+    const int seg0 = r.seg0, bag0 = r.t * a.B, out0 = r.out0;
+    const uint32_t key0 = (uint32_t)((uint64_t)r.t * (uint64_t)a.N);
+    const bool hot_first = r.hot_row < r.base;
+    auto write = [&](int j, uint32_t key, int pos, int bag, uint32_t u) {
+      o.keys[j] = key;
+      o.perm[j] = pos;
+      if (o.perm_out) o.perm_out[j] = pos;
+      o.uidx[j] = (int32_t)u;
+      o.sbag[j] = bag;
+    };
+    {
+      const uint32_t base = key0 + r.base;
+      uint32_t u_next = r.before + (hot_first && r.hot > 0) + __shfl_sync(0xffffffffu, inc - (lane == 0 ? heads : 0u), 0);
 #pragma unroll 4
-  for (int j = i0 + lane; j < iend; j += 32) {
-    const int pay = j < q ? order[j] : 0;
-    const uint32_t k = okey[pay];
-    const int pos = seg0 + opos[pay];
-    const int bag = (int)bag0 + obag[pay];
-    const bool head = head_at(j, k);
-    const uint32_t m = __ballot_sync(0xffffffffu, head);
-    const uint32_t u = u_next + __popc(m & (0xffffffffu >> (31 - lane))) - 1u;
-    u_next += __popc(m);
-    if (j < q) {
-      const uint32_t key = key0 + k;
-      o.keys[out0 + j] = key;
-      o.perm[out0 + j] = pos;
-      if (o.perm_out) o.perm_out[out0 + j] = pos;
-      o.uidx[out0 + j] = (int32_t)u;
-      o.sbag[out0 + j] = bag;
-      // (u < L unless another table's offsets are malformed; then the fallback writes all of this again)
-      if (head && (int64_t)u < o.L) put_unique(o, u, key, out0 + j);
+      for (int j = i0 + lane; j < iend; j += 32) {
+        const int pay = j < q ? order[j] : 0;
+        const uint32_t k = okey[pay];
+        const int pos = seg0 + opos[pay];
+        const int bag = bag0 + obag[pay];
+        const bool head = head_at(j, k);
+        const uint32_t m = __ballot_sync(0xffffffffu, head);
+        const uint32_t u = u_next + __popc(m & (0xffffffffu >> (31 - lane))) - 1u;
+        u_next += __popc(m);
+        if (j < q) {
+          write(out0 + j, base + k, pos, bag, u);
+          // (u < L unless another table's offsets are malformed; then the fallback writes all of this again)
+          if (head && (int64_t)u < o.L) put_unique(o, u, base + k, out0 + j);
+        }
+      }
     }
-  }
-  if (id == a.T * a.C - 1 && tid == 0) {
-    put_segment_end(o, min(u0 + mine_u, (uint32_t)o.L), o.L);
-    finish_unique(o, u0 + mine_u);
-  }
+    if (r.hot > 0) {
+      const int n = r.seg1 - seg0, first = hot_first ? out0 - r.hot : out0 + q;
+      const uint32_t key = key0 + r.hot_row, u = hot_first ? r.before : r.before + r.mine - 1u;
+      WalkStart start(a, r, n);
+      uint32_t seen = 0;
+      __syncthreads();                                     // everybody is done with what the block kept and with the counters
+      walk_table(a, r, crow, cbag, n, start, r.hot_row, 1u, kNoRow, r.hot, seen,
+                 [&](int, int i, uint32_t, int position, int bag) {
+                   opos[i] = (uint16_t)position;
+                   obag[i] = (uint16_t)bag;
+                 },
+                 [&](int done, int count) {
+                   for (int i = tid; i < count; i += kBsThreads) write(first + done + i, key, seg0 + opos[i], bag0 + obag[i], u);
+                 });
+      if (tid == 0 && (int64_t)u < o.L) put_unique(o, u, key, first);
+    }
+    if (r.id == r.total - 1 && tid == 0) {
+      put_segment_end(o, min(r.before + r.mine, (uint32_t)o.L), o.L);
+      finish_unique(o, r.before + r.mine);
+    }
+  } while (false);
   if (a.serial_fallback) {
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_scalar[0] = (uint32_t)atomicAdd(a.ticket + 1, 1);
+    if (tid == 0) r.id = (uint32_t)atomicAdd(a.ticket + 1, 1);
     __syncthreads();
-    if ((int)s_scalar[0] != (int)gridDim.x - 1) return;
+    if (r.id != gridDim.x - 1) return;
     __threadfence();
     if (*reinterpret_cast<volatile int32_t*>(a.fallback) != 0)
       tiled_sort_items<kBsThreads>(tiled, reinterpret_cast<uint32_t*>(bs_raw), 1);
@@ -1468,60 +1626,56 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, cons
 // Closes an empty sort.
 __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_for_previous_kernel(); finish_unique(o, 0u); }
 
-// Whether the bucket sort takes a problem, and how it cuts it.  Every further range reads the index list once more and holds
-// an SM, so a table gets the fewest ranges that hold its lookups when one row draws 22 % of them (a Zipf exponent of 1.2
-// over a few thousand rows; more skew than that on a long table takes the tiled sort): four replicas of the ordinary model
-// 478 us a round with two ranges, 499 with three, 508 with four.  Few tables are cut finer, down to 5500 lookups a
-// range, while that takes no more than a quarter of the SMs (5 tables of 9000 lookups: 91 -> 79 us for lookup and update).
-static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, BucketSort* a, int* nb) {
+// Whether the bucket sort takes a problem, how many lookups it gives a range, and the most ranges there can be, whatever the
+// tables' lengths: a block for each.  Every further range reads the index list once more and holds an SM, so a table gets as
+// few ranges as hold its lookups.  Few tables are cut finer, down to 5500 lookups a range, while that takes no more than a
+// quarter of the SMs (5 tables of 9000 lookups: 91 -> 79 us for lookup and update).
+static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, BucketSort* a, int64_t* blocks, int* nb) {
   const int64_t avg = (L + T - 1) / T;
-  if (B > 65535) return false;                             // bag numbers, plus one, take 16 bits
-  constexpr int64_t kFull = 14000;                         // a little below the least capacity (digits of 10 bits)
-  const int64_t hot = avg > kFull ? avg * 22 / 100 : 0;
-  if (hot >= kFull * 4 / 5) return false;
-  int64_t C = (avg - hot + kFull - hot - 1) / (kFull - hot);
+  if (B > 65535 || avg > 44000) return false;              // bag numbers, plus one, take 16 bits
+  int64_t C = (avg + kBsRange - 1) / kBsRange;
   const int64_t fine = (avg + 5499) / 5500, room = num_sms() / 4 / T;
-  if (C < fine && C < room) C = fine < room ? fine : room;
-  // more than one wave of blocks: as many ranges as two waves take (40 tables of 33 500 lookups: 93 us with 4 ranges, 79 with 7)
-  if (C * T > num_sms() && C < 2 * num_sms() / T) C = 2 * num_sms() / T < kBsMaxBuckets ? 2 * num_sms() / T : kBsMaxBuckets;
-  if (C > kBsMaxBuckets) return false;
+  a->per_range = kBsRange;
+  if (C < fine && C < room) {
+    C = fine < room ? fine : room;
+    if (C > kBsMaxBuckets) C = kBsMaxBuckets;
+    a->per_range = (int)(avg * 115 / 100 / C);             // tables a little longer than the average get no further range
+  }
   if (C < 1) C = 1;
-  if (C > N) C = N;
-  a->rows_per = (int)((N + C - 1) / C);
-  a->C = (int)((N + a->rows_per - 1) / a->rows_per);       // no empty range
   a->T = T; a->B = B; a->N = N;
+  a->ranges = T > kBsThreads ? (int)C : 0;
   int bits = 1;
-  while (((uint64_t)(a->rows_per - 1) >> bits) != 0) ++bits;
-  a->passes = (bits + kBsDigit - 1) / kBsDigit;
-  *nb = (bits + a->passes - 1) / a->passes;
+  while (((uint64_t)(N - 1) >> bits) != 0) ++bits;
+  const int passes = (bits + kBsDigit - 1) / kBsDigit;
+  *nb = (bits + passes - 1) / passes;                      // as few passes as a range of all rows takes (most take fewer bits)
   if (*nb < 5) *nb = 5;                                    // the in-block scan wants at least 32 bins
-  const int cap = bs_cap(*nb);
-  a->cap = L < cap ? (int)((L + 31) & ~(int64_t)31) : cap; // small problems leave shared memory to others
+  a->cap = L < kBsCap ? (int)((L + 31) & ~(int64_t)31) : kBsCap;   // small problems leave shared memory to others
+  *blocks = a->ranges > 0 ? T * C : T + L / a->per_range;
   return true;
 }
 
 template <int NB>
-static ss_status launch_bucket_sort_nb(const BucketSort& a, const TiledSort& t, cudaStream_t st) {
+static ss_status launch_bucket_sort_nb(const BucketSort& a, const TiledSort& t, int64_t blocks, cudaStream_t st) {
   static bool attr_set[64];
   int dev = 0;
   SS_CUDA(cudaGetDevice(&dev));
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    SS_CUDA(cudaFuncSetAttribute(bucket_sort_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs_smem(bs_cap(NB), NB)));
+    SS_CUDA(cudaFuncSetAttribute(bucket_sort_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs_smem(kBsCap, NB)));
     attr_set[dev] = true;
   }
   SS_TIMED("bucket_sort_kernel", st);
-  launch_dependent(bucket_sort_kernel<NB>, a.T * a.C, kBsThreads, bs_smem(a.cap, NB), st, a, t);
+  launch_dependent(bucket_sort_kernel<NB>, (unsigned)blocks, kBsThreads, bs_smem(a.cap, NB), st, a, t);
   SS_LAUNCH_OK();
   return SS_OK;
 }
-static ss_status launch_bucket_sort(const BucketSort& a, const TiledSort& t, int nb, cudaStream_t st) {
+static ss_status launch_bucket_sort(const BucketSort& a, const TiledSort& t, int64_t blocks, int nb, cudaStream_t st) {
   switch (nb) {
-    case 5: return launch_bucket_sort_nb<5>(a, t, st);
-    case 6: return launch_bucket_sort_nb<6>(a, t, st);
-    case 7: return launch_bucket_sort_nb<7>(a, t, st);
-    case 8: return launch_bucket_sort_nb<8>(a, t, st);
-    case 9: return launch_bucket_sort_nb<9>(a, t, st);
-    default: return launch_bucket_sort_nb<10>(a, t, st);
+    case 5: return launch_bucket_sort_nb<5>(a, t, blocks, st);
+    case 6: return launch_bucket_sort_nb<6>(a, t, blocks, st);
+    case 7: return launch_bucket_sort_nb<7>(a, t, blocks, st);
+    case 8: return launch_bucket_sort_nb<8>(a, t, blocks, st);
+    case 9: return launch_bucket_sort_nb<9>(a, t, blocks, st);
+    default: return launch_bucket_sort_nb<10>(a, t, blocks, st);
   }
 }
 
@@ -1615,15 +1769,16 @@ static ss_status bwd_impl(bool do_sort, bool do_apply, float* tables, float* row
     ts.tile_heads = reinterpret_cast<uint32_t*>(ws + p.off_heads);
     ts.ctl = ctl + kCtlTiled; ts.passes = p.passes; ts.digit_bits = p.digit_bits; ts.bins = p.bins; ts.out = out;
     BucketSort bs{};
+    int64_t blocks = 0;
     int nb = 0;
-    const bool bucket = plan_bucket_sort(T, N, B, L, &bs, &nb);
-    stt = clear_words(ctl, kCtlCounts + (bucket ? T * bs.C : 0), cs);
+    const bool bucket = plan_bucket_sort(T, N, B, L, &bs, &blocks, &nb);
+    stt = clear_words(ctl, kCtlCounts + (bucket ? T * kBsMaxBuckets : 0), cs);
     if (stt != SS_OK) return stt;
     if (bucket) {
       bs.indices = indices; bs.offsets = offsets;
       bs.fallback = ctl + kCtlFallback; bs.ticket = ctl + kCtlTicket; bs.counts = reinterpret_cast<uint32_t*>(ctl + kCtlCounts);
       bs.serial_fallback = L <= bs.cap;                    // no range can be too full: only malformed input takes the fallback
-      stt = launch_bucket_sort(bs, ts, nb, cs);
+      stt = launch_bucket_sort(bs, ts, blocks, nb, cs);
       if (stt != SS_OK) return stt;
       ts.run_if = bs.fallback;
     }

@@ -1,6 +1,7 @@
-"""The sort / unique half of the embedding backward where its cuts lie: bucket ranges, chunk and round edges, a range that
-overflows its block (the tiled passes take over), one row, one table, malformed input.  Integer outputs are bit-exact
-against a stable argsort of the keys."""
+"""The sort / unique half of the embedding backward where its cuts lie: bucket ranges, chunk and round edges, popular rows
+that are neighbours, a row too popular for a block, uneven tables, one row, one table, malformed input.  Integer outputs are
+bit-exact against a stable argsort of the keys; and the ranges hold whatever the rows' distribution is, so that the tiled
+passes (for long tables) never have to sort a problem again that the bucket sort was given."""
 import numpy as np
 import pytest
 import torch
@@ -20,6 +21,7 @@ def _sort(T, N, B, idx, off):
     ss.ss_embbag_bwd_sort(T, N, 8, di, do, B, L, ws, uniq, seg, perm, num, st)
     torch.cuda.synchronize()
     U = int(num.item())
+    _sort.fell_back = int(ws[-(-(32 + 32 * T) // 256) * -256:][:4].view(torch.int32).item())   # first control word of the workspace
     return uniq.cpu().numpy()[:U], seg.cpu().numpy()[:U + 1], perm.cpu().numpy()[:L], int(st.item())
 
 
@@ -28,7 +30,7 @@ def _offsets(lens):
 
 
 def _check(T, N, B, lens, row_of):
-    """lens [T*B]; row_of(rng, n) -> n row ids of a table."""
+    """lens [T*B]; row_of(rng, n) -> n row ids."""
     rng = np.random.default_rng(T * 1000 + N + B)
     off = _offsets(lens)
     table_of = np.repeat(np.arange(T * B) // B, lens)
@@ -37,14 +39,19 @@ def _check(T, N, B, lens, row_of):
     perm = np.argsort(keys, kind="stable")
     uniq, first = np.unique(keys, return_index=True)
     got_u, got_s, got_p, st = _sort(T, N, B, idx, off)
-    assert st == 0
+    assert st == 0 and _sort.fell_back == 0
     assert np.array_equal(got_p, perm)
     assert np.array_equal(got_u, uniq)
     assert np.array_equal(got_s, np.concatenate([np.flatnonzero(np.diff(keys[perm], prepend=-1)), [idx.size]]))
 
 
 UNIFORM = lambda N: (lambda rng, n: rng.integers(0, N, n))
-HOT_LOW = lambda N: (lambda rng, n: np.minimum(rng.zipf(1.3, n) - 1, N - 1))     # popular rows have low ids: one full range
+HOT_LOW = lambda N: (lambda rng, n: np.minimum(rng.zipf(1.3, n) - 1, N - 1))     # popular rows have low ids
+
+
+def ONE_ROW(share, at):
+    """One row, at a fraction of the table, draws a share of the lookups (an id that stands for "missing")."""
+    return lambda N: (lambda rng, n: np.where(rng.random(n) < share, int(at * (N - 1)), rng.integers(0, N, n)))
 
 
 @pytest.mark.parametrize("T,N,B,bag,rows", [
@@ -52,8 +59,14 @@ HOT_LOW = lambda N: (lambda rng, n: np.minimum(rng.zipf(1.3, n) - 1, N - 1))    
     (2, 1000, 64, 128, UNIFORM),                     # 8192 lookups a table: exactly one chunk, bags longer than a warp's share
     (2, 1000, 8193, 1, UNIFORM),                     # one lookup more: two chunks, two ranges
     (4, 999_983, 2048, 9, UNIFORM),                  # three ranges of 18 and 19 bits
-    (3, 100_003, 6000, 8, UNIFORM), (3, 100_003, 6000, 8, HOT_LOW),     # six ranges; nearly all lookups in one: tiled passes
-    (2, 50_000, 2000, 10, HOT_LOW),                  # nearly all lookups in one range, which holds them
+    (3, 100_003, 6000, 8, UNIFORM), (3, 100_003, 6000, 8, HOT_LOW),
+    (2, 50_000, 2000, 10, HOT_LOW),
+    (40, 1_000_000, 2048, 10, HOT_LOW),              # two ranges a table, most lookups in the first thousand rows
+    (20, 1_000_000, 2048, 10, ONE_ROW(0.9, 0.3)),    # 18 400 lookups of a row: more than a block sorts
+    (20, 500, 2048, 16, ONE_ROW(0.5, 0.0)), (20, 500, 2048, 16, ONE_ROW(0.97, 1.0)), (20, 3, 2048, 16, ONE_ROW(1.0, 1.0)),
+    (20, 1, 2048, 16, UNIFORM),
+    (4, 1_000_000, 8192, 5, ONE_ROW(0.6, 0.5)),      # seven ranges
+    (1030, 50, 60, 1, UNIFORM),                      # more tables than a block has threads
     (1, 300_000, 65_536, 1, UNIFORM), (1, 300_000, 40_000, 2, UNIFORM),   # beyond the bucket sort: tiled passes
 ])
 def test_sort_matches_a_stable_argsort(T, N, B, bag, rows):
@@ -64,6 +77,14 @@ def test_sort_of_uneven_tables_and_empty_bags():
     rng = np.random.default_rng(5)
     lens = np.concatenate([np.zeros(500, int), rng.integers(0, 4, 500), rng.integers(0, 90, 500), np.full(500, 1)])
     _check(4, 12_345, 500, lens, UNIFORM(12_345))
+
+
+@pytest.mark.parametrize("rows", [UNIFORM, HOT_LOW, ONE_ROW(0.8, 0.6)])
+def test_sort_of_tables_of_very_different_lengths(rows):
+    """Ranges follow each table's own lookups: an empty table, 60 000 lookups beside 2000."""
+    B, N = 2000, 200_000
+    lens = np.concatenate([np.full(B, k) for k in (1, 30, 0, 7, 1, 12, 1, 1, 6, 1, 25, 2)])
+    _check(12, N, B, lens, rows(N))
 
 
 @pytest.mark.parametrize("B,bag", [(40, 2), (3000, 9)])
