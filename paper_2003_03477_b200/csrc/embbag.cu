@@ -614,11 +614,13 @@ tiled_sort_kernel(const __grid_constant__ TiledSort a) {
 // Blocks take their ranges from a ticket, so the counts a block waits for come from blocks that are running.  There are as
 // many blocks as tables of any lengths could need; those without a range leave at once.
 //
-// The cut follows the data.  A table gets a range per `per_range` of its own lookups, and the ranges hold about equally
-// many: their edges are quantiles of 2048 lookups spread over the table, which every block of the table reads alike.  So it
-// does not matter whether popular rows are scattered or neighbours, or one table is longer than another.  A popular row on
-// an edge goes to the side that has less of it; where a range is too full all the same, because its first or last row draws
-// so much, that row is not sorted but copied out, in order, by a second walk over the index list.
+// The cut follows the data, so it does not matter whether popular rows are scattered or neighbours, or one table is longer
+// than another.  A table gets a range per `per_range` of its own lookups: equal slices of its rows at first.  While a block
+// collects its slice it counts all slices of the table, and if one of them does not fit into a block, every block of the
+// table comes to know that; they collect again, ranges whose edges are quantiles of 2048 lookups spread over the table,
+// which they all read alike.  A popular row on an edge goes to the side that has less of it; where a range is too full all
+// the same, because its first or last row draws so much, that row is not sorted but copied out, in order, by one more walk
+// over the index list.  (Quantiles in the first place, or samples that tell whether slices will do, cost 2-4 us a call.)
 // What bounds it is instruction issue and the latency of a block's rounds.
 //
 // A block that cannot take the path (a range with more lookups than `cap` after all, a table of more than 65536, offsets
@@ -736,6 +738,8 @@ struct BucketRange {
   int t, c, ranges, seg0, seg1;                            // its table, its number there, how many there are, the table's segment
   uint32_t edge[2], rank[2];                               // while the edges are looked for
   uint32_t base, span, hot_row;                            // rows [base, base + span) are sorted, one beside them may be copied out
+  uint32_t edges[kBsMaxBuckets - 1], part[kBsMaxBuckets - 1][kBsWarps];   // rows; lookups of rows before them, per warp
+  int n_edges, lt[kBsMaxBuckets - 1];                      // and in all
   int kept, hot, out0;                                     // lookups sorted and copied out, where the sorted ones go
   uint32_t mine, before;                                   // distinct rows of this range and of those before it
 };
@@ -774,7 +778,7 @@ __device__ __forceinline__ void select_two(BucketRange& r, uint32_t* hist, const
 }
 
 constexpr uint32_t kNoRow = 0xffffffffu;                   // no row id is that large
-// What a thread has in flight before a walk: the first chunk of the index list, the offsets of bag `tid`.
+// What a thread has in flight before a walk: the first chunk of the index list (kNoRow beyond its end), the offsets of bag `tid`.
 struct WalkStart {
   uint32_t next[8];
   int l, h;
@@ -784,18 +788,18 @@ struct WalkStart {
     l = h = 0;
     if (tid < a.B) { l = off[tid]; h = off[tid + 1]; }
 #pragma unroll
-    for (int k = 0; k < 8; ++k) next[k] = tid + k * kBsThreads < n ? (uint32_t)__ldg(a.indices + r.seg0 + tid + k * kBsThreads) : 0u;
+    for (int k = 0; k < 8; ++k) next[k] = tid + k * kBsThreads < n ? (uint32_t)__ldg(a.indices + r.seg0 + tid + k * kBsThreads) : kNoRow;
   }
 };
 
 // Walks the index list of table r.t, n long, and hands the lookups of rows [from, from + rows) to put(number, number in the
-// chunk, row, position, bag), in order, and after each chunk their numbers to flush(first, count); their count, or -1: more
-// than `limit`, or malformed.  Per thread, `seen` counts the lookups of rows before `from`, and in its upper half those of
-// row `hot`.  The list goes through shared memory so that its loads are coalesced; a chunk's loads are in flight while the
-// chunk before is worked on.
+// chunk, row, position, bag), in order, and after each chunk their numbers to flush(first, count); their count, or -1: the
+// list is malformed.  Per thread, byte j % 4 of seen[j / 4] counts the lookups of rows before r.edges[j] (a thread looks at
+// 64 positions at most).  The list goes through shared memory so that its loads are coalesced; a chunk's loads are in flight
+// while the chunk before is worked on.
 template <typename Put, typename Flush>
 __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, uint32_t* crow, uint16_t* cbag, int n, WalkStart& start,
-                                          uint32_t from, uint32_t rows, uint32_t hot, int limit, uint32_t& seen, Put put, Flush flush) {
+                                          uint32_t from, uint32_t rows, int n_edges, uint32_t (&seen)[2], Put put, Flush flush) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int seg0 = r.seg0, seg1 = seg0 + n;
   const int32_t* off = a.offsets + (int64_t)r.t * a.B;
@@ -821,7 +825,7 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int p = p0 + kBsChunk + tid + k * kBsThreads;
-      start.next[k] = p < n ? (uint32_t)__ldg(a.indices + seg0 + p) : 0u;
+      start.next[k] = p < n ? (uint32_t)__ldg(a.indices + seg0 + p) : kNoRow;
     }
     __syncthreads();
     const uint4 r0 = *reinterpret_cast<const uint4*>(crow + 8 * tid), r1 = *reinterpret_cast<const uint4*>(crow + 8 * tid + 4);
@@ -829,14 +833,15 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
     int mine = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const bool in = w0 + k < p1;
-      if (in && row[k] >= (uint32_t)a.N) bad = 1;          // one unsigned compare: negative indices are huge
-      mine += in && row[k] - from < rows;
-      seen += in && row[k] < from;
+      if (row[k] >= (uint32_t)a.N && w0 + k < p1) bad = 1; // one unsigned compare: negative indices are huge
+      mine += row[k] - from < rows;
     }
-    if (hot != kNoRow) {
+    for (int j = 0; j < n_edges; ++j) {
+      const uint32_t edge = r.edges[j];
+      uint32_t c = 0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) seen += w0 + k < p1 && row[k] == hot ? 0x10000u : 0u;   // at most 64 positions a thread
+      for (int k = 0; k < 8; ++k) c += row[k] < edge;
+      if (j < 4) seen[0] += c << 8 * j; else seen[1] += c << 8 * (j - 4);
     }
     if (__syncthreads_or(bad)) return -1;
     const uint4 mk = *reinterpret_cast<const uint4*>(cbag + 8 * tid);
@@ -861,7 +866,6 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
       if (lane >= d) { ws += u; wm = max(wm, v); }
     }
     const int chunk = (int)__shfl_sync(0xffffffffu, ws, 31);
-    if (kept + chunk > limit) return -1;
     int at = kept + (int)(__shfl_sync(0xffffffffu, ws - ws0, warp) + sum) - mine;
     uint32_t bag = __shfl_up_sync(0xffffffffu, mx, 1);
     if (lane == 0) bag = 0;
@@ -871,7 +875,7 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       bag = max(bag, (k & 1) ? mw[k >> 1] >> 16 : mw[k >> 1] & 0xffffu);
-      if (w0 + k < p1 && row[k] - from < rows) {
+      if (row[k] - from < rows) {
         put(at, at - kept, row[k], w0 + k, (int)bag - 1);
         ++at;
       }
@@ -881,6 +885,59 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
     kept += chunk;
   }
   return kept;
+}
+
+__device__ __forceinline__ void write_sorted(const SortOut& o, int j, uint32_t key, int pos, int bag, uint32_t u) {
+  o.keys[j] = key;
+  o.perm[j] = pos;
+  if (o.perm_out) o.perm_out[j] = pos;
+  o.uidx[j] = (int32_t)u;
+  o.sbag[j] = bag;
+}
+
+// The range's rows by quantiles of samples: r.base, r.span, r.hot_row, and the rows whose lookups the walk is to count.
+__device__ __noinline__ void recut(const BucketSort& a, BucketRange& r, uint32_t* hist) {
+  const int tid = threadIdx.x, n = r.seg1 - r.seg0, c = r.c, C = r.ranges;
+  uint32_t sample[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) sample[i] = min((uint32_t)__ldg(a.indices + r.seg0 + (((2 * tid + i) * n) >> 11)), (uint32_t)a.N - 1u);
+  select_two(r, hist, sample, max(1, 32 - __clz((uint32_t)a.N - 1u)), c * kBsSamples / C, min((c + 1) * kBsSamples / C, kBsSamples - 1));
+  const uint32_t lo = c > 0 ? r.edge[0] : 0u, hi = c < C - 1 ? r.edge[1] : (uint32_t)a.N;
+  auto count = [&](uint32_t from, uint32_t rows) {         // samples of rows [from, from + rows)
+    return __syncthreads_count(sample[0] - from < rows) + __syncthreads_count(sample[1] - from < rows);
+  };
+  // what a block holds, less five standard deviations of the samples' share (1 / 18 = 2.5 / sqrt(2048)), in samples
+  uint32_t hot = kNoRow;
+  if (count(lo, hi - lo) > (int)((int64_t)(a.cap - n / 18) * kBsSamples / n)) hot = count(lo, 1u) >= count(hi - 1u, 1u) ? lo : hi - 1u;
+  if (tid == 0) {
+    r.base = lo + (hot == lo);
+    r.span = hi - r.base - (hot != lo && hot != kNoRow);
+    r.hot_row = hot;
+    r.edges[0] = r.base; r.edges[1] = hot; r.edges[2] = hot + 1u;
+    r.n_edges = hot == kNoRow ? 1 : 3;
+  }
+}
+
+// Outputs of the row of a range that is not sorted.  Out of line: few ranges have one, and inside the kernel its registers
+// cost every range (26 tables of 21 500 lookups 43 -> 45 us).
+__device__ __noinline__ void copy_row(const BucketSort& a, const SortOut& o, BucketRange& r, uint16_t* opos, uint16_t* obag,
+                                      uint32_t* crow, uint16_t* cbag) {
+  const int tid = threadIdx.x, seg0 = r.seg0, n = r.seg1 - seg0, bag0 = r.t * a.B;
+  const bool before = r.hot_row < r.base;                  // the sorted rows
+  const int first = before ? r.out0 - r.hot : r.out0 + r.kept;
+  const uint32_t key = (uint32_t)((uint64_t)r.t * (uint64_t)a.N) + r.hot_row, u = before ? r.before : r.before + r.mine - 1u;
+  WalkStart start(a, r, n);
+  uint32_t unused[2] = {0u, 0u};
+  __syncthreads();                                         // everybody is done with what the block kept and with the counters
+  walk_table(a, r, crow, cbag, n, start, r.hot_row, 1u, 0, unused,
+             [&](int, int i, uint32_t, int position, int bag) {
+               opos[i] = (uint16_t)position;
+               obag[i] = (uint16_t)bag;
+             },
+             [&](int done, int count) {
+               for (int i = tid; i < count; i += kBsThreads) write_sorted(o, first + done + i, key, seg0 + opos[i], bag0 + obag[i], u);
+             });
+  if (tid == 0 && (int64_t)u < o.L) put_unique(o, u, key, first);
 }
 
 template <int NB>                                          // digit bits, 5..kBsDigit
@@ -901,22 +958,55 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   do {                                                     // (a break: nothing to do for this block)
     // ---- how many ranges every table has, by its lookups, and which range is this block's; thread t looks after table t
-    if (a.ranges == 0) {
-      constexpr int kBad = 1 << 20;                        // more than all ranges
-      int first = 0, last = 0, mine = 0;
-      if (tid < a.T) {
-        first = a.offsets[(int64_t)tid * a.B];
-        last = a.offsets[(int64_t)(tid + 1) * a.B];
+    constexpr int kBad = 1 << 20;                          // more than all ranges
+    auto ranges_of = [&](int t, int first, int last) {
+      return sound_table(a, o.L, t, first, last) ? max(1, min(kBsMaxBuckets, (last - first + a.per_range - 1) / a.per_range)) : kBad;
+    };
+    auto take = [&](int id, int t, int end, int ranges, int first, int last) {
+      if (id < end && id >= end - ranges) { r.t = t; r.c = id - (end - ranges); r.ranges = ranges; r.seg0 = first; r.seg1 = last; }
+    };
+    if (a.ranges == 0 && a.T <= 64) {
+      if (warp == 0) {                                     // one warp, two tables a lane: the others issue nothing meanwhile
+        int first[2] = {0, 0}, last[2] = {0, 0}, ranges[2] = {0, 0}, id = 0;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int t = lane + 32 * i;
+          if (t < a.T) { first[i] = a.offsets[(int64_t)t * a.B]; last[i] = a.offsets[(int64_t)(t + 1) * a.B]; }
+        }
+        if (lane == 0) id = atomicAdd(a.ticket, 1);
+        int end = 0;
+        id = __shfl_sync(0xffffffffu, id, 0);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int t = lane + 32 * i;
+          if (t < a.T) ranges[i] = ranges_of(t, first[i], last[i]);
+          int upto = ranges[i];
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, upto, d);
+            if (lane >= d) upto += x;
+          }
+          take(id, t, end + upto, ranges[i], first[i], last[i]);
+          end += __shfl_sync(0xffffffffu, upto, 31);
+        }
+        if (lane == 0) {
+          r.id = (uint32_t)id; r.total = (uint32_t)end;
+          if (end >= kBad) atomicOr(a.fallback, 1);
+        }
       }
+      __syncthreads();
+      if (r.id >= r.total || r.total >= (uint32_t)kBad) break;
+    } else if (a.ranges == 0) {
+      int first = 0, last = 0, ranges = 0;
+      if (tid < a.T) { first = a.offsets[(int64_t)tid * a.B]; last = a.offsets[(int64_t)(tid + 1) * a.B]; }
       if (tid == 0) r.id = (uint32_t)atomicAdd(a.ticket, 1);
-      if (tid < a.T)
-        mine = sound_table(a, o.L, tid, first, last) ? max(1, min(kBsMaxBuckets, (last - first + a.per_range - 1) / a.per_range)) : kBad;
-      const int end = (int)block_scan<kBsThreads>((uint32_t)mine, r.w), id = (int)r.id;
+      if (tid < a.T) ranges = ranges_of(tid, first, last);
+      const int end = (int)block_scan<kBsThreads>((uint32_t)ranges, r.w);
       if (tid == kBsThreads - 1) {
         r.total = (uint32_t)end;
         if (end >= kBad) atomicOr(a.fallback, 1);
       }
-      if (id < end && id >= end - mine) { r.t = tid; r.c = id - (end - mine); r.ranges = mine; r.seg0 = first; r.seg1 = last; }
+      take((int)r.id, tid, end, ranges, first, last);
       __syncthreads();
       if (r.id >= r.total || r.total >= (uint32_t)kBad) break;
     } else {
@@ -930,54 +1020,55 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
       __syncthreads();
     }
     // ---- the range's rows, and its lookups into shared memory
-    {
-      const bool sound = sound_table(a, o.L, r.t, r.seg0, r.seg1);
+    const bool sound = sound_table(a, o.L, r.t, r.seg0, r.seg1);
+    for (int attempt = 0;; ++attempt) {
       const int n = sound ? r.seg1 - r.seg0 : 0, C = r.ranges;
-      uint32_t sample[2] = {0u, 0u};
-      if (C > 1 && n > 0) {
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-          sample[i] = min((uint32_t)__ldg(a.indices + r.seg0 + (((2 * tid + i) * n) >> 11)), (uint32_t)a.N - 1u);
-      }
       WalkStart start(a, r, n);
-      uint32_t lo = 0, hi = (uint32_t)a.N, hot = kNoRow;   // hot: the row that is copied out
-      if (C > 1 && n > 0) {
-        const int c = r.c, bits = max(1, 32 - __clz((uint32_t)a.N - 1u));
-        select_two(r, okey, sample, bits, c * kBsSamples / C, min((c + 1) * kBsSamples / C, kBsSamples - 1));
-        if (c > 0) lo = r.edge[0];
-        if (c < C - 1) hi = r.edge[1];
-        auto count = [&](uint32_t from, uint32_t rows) {   // samples of rows [from, from + rows)
-          return __syncthreads_count(sample[0] - from < rows) + __syncthreads_count(sample[1] - from < rows);
-        };
-        // five standard deviations of the samples' share below what the block can hold (1 / 18 = 2.5 / sqrt(2048))
-        if ((int64_t)count(lo, hi - lo) * n > (int64_t)(cap - n / 18) * kBsSamples) hot = count(lo, 1u) >= count(hi - 1u, 1u) ? lo : hi - 1u;
+      if (attempt > 0) {
+        recut(a, r, okey);
+      } else if (tid < kBsMaxBuckets) {
+        const uint32_t width = ((uint32_t)a.N + C - 1u) / C, edge = min((tid + 1u) * width, (uint32_t)a.N);
+        if (tid < kBsMaxBuckets - 1) r.edges[tid] = edge;
+        if (tid == r.c) { r.base = min(tid * width, (uint32_t)a.N); r.span = edge - r.base; r.hot_row = kNoRow; r.n_edges = C - 1; }
       }
-      const uint32_t base = lo + (hot == lo), span = hi - base - (hot != lo && hot != kNoRow);
-      uint32_t seen = 0;
-      const int kept = walk_table(a, r, crow, cbag, n, start, base, span, hot, cap, seen,
+      __syncthreads();
+      const uint32_t base = r.base;
+      const int n_edges = r.n_edges;
+      uint32_t seen[2] = {0u, 0u};
+      const int kept = walk_table(a, r, crow, cbag, n, start, base, r.span, n_edges, seen,
                                   [&](int at, int, uint32_t row, int position, int bag) {
+                                    if (at >= cap) return;
                                     okey[at] = row - base;
                                     opos[at] = (uint16_t)position;
                                     obag[at] = (uint16_t)bag;
                                   }, [](int, int) {});
-      const bool ok = sound && kept >= 0;
-      if (!ok && tid == 0) atomicOr(a.fallback, 1);
-      const int q = ok ? kept : 0;
-      // pads of the last round: the largest digits and the last places, so every stable pass leaves them at the end
-      __syncthreads();
-      if (tid < ((q + 31) & ~31) - q) okey[q + tid] = 0xffffffffu;
-      const uint32_t below = __reduce_add_sync(0xffffffffu, seen & 0xffffu), n_hot = __reduce_add_sync(0xffffffffu, seen >> 16);
-      if (lane == 0) { r.w[warp] = below; r.m[warp] = n_hot; }
-      __syncthreads();
-      if (warp == 0) {
-        const int all_below = (int)__reduce_add_sync(0xffffffffu, r.w[lane]), all_hot = (int)__reduce_add_sync(0xffffffffu, r.m[lane]);
-        if (lane == 0) {
-          r.base = base; r.span = span; r.hot_row = hot; r.kept = q;
-          r.hot = ok ? all_hot : 0;
-          r.out0 = r.seg0 + all_below;
-        }
+      for (int j = 0; j < n_edges; ++j) {
+        const uint32_t c = __reduce_add_sync(0xffffffffu, (seen[j >> 2] >> 8 * (j & 3)) & 0xffu);
+        if (lane == 0) r.part[j][warp] = c;
       }
       __syncthreads();
+      if (warp < n_edges) {
+        const int c = (int)__reduce_add_sync(0xffffffffu, r.part[warp][lane]);
+        if (lane == 0) r.lt[warp] = c;
+      }
+      __syncthreads();
+      int fullest = kept;                                  // of the range, or of all slices of the table
+      if (attempt == 0) {
+        for (int c = 0; c < C; ++c) fullest = max(fullest, (c < C - 1 ? r.lt[c] : n) - (c > 0 ? r.lt[c - 1] : 0));
+        if (kept >= 0 && C > 1 && fullest > cap) continue;
+      }
+      const bool ok = sound && kept >= 0 && fullest <= cap;
+      const int q = ok ? kept : 0;
+      // pads of the last round: the largest digits and the last places, so every stable pass leaves them at the end
+      if (tid < ((q + 31) & ~31) - q) okey[q + tid] = 0xffffffffu;
+      if (tid == 0) {
+        if (!ok) atomicOr(a.fallback, 1);
+        r.kept = q;
+        r.hot = ok && n_edges == 3 && attempt > 0 ? r.lt[2] - r.lt[1] : 0;
+        r.out0 = r.seg0 + (attempt > 0 ? r.lt[0] : (r.c > 0 ? r.lt[r.c - 1] : 0));
+      }
+      __syncthreads();
+      break;
     }
     // ---- sort
     const int q = r.kept, q32 = (q + 31) & ~31;
@@ -1022,17 +1113,9 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
     // ---- outputs: the sorted rows, and the row copied out before or behind them
     const int seg0 = r.seg0, bag0 = r.t * a.B, out0 = r.out0;
     const uint32_t key0 = (uint32_t)((uint64_t)r.t * (uint64_t)a.N);
-    const bool hot_first = r.hot_row < r.base;
-    auto write = [&](int j, uint32_t key, int pos, int bag, uint32_t u) {
-      o.keys[j] = key;
-      o.perm[j] = pos;
-      if (o.perm_out) o.perm_out[j] = pos;
-      o.uidx[j] = (int32_t)u;
-      o.sbag[j] = bag;
-    };
     {
       const uint32_t base = key0 + r.base;
-      uint32_t u_next = r.before + (hot_first && r.hot > 0) + __shfl_sync(0xffffffffu, inc - (lane == 0 ? heads : 0u), 0);
+      uint32_t u_next = r.before + (r.hot > 0 && r.hot_row < r.base) + __shfl_sync(0xffffffffu, inc - (lane == 0 ? heads : 0u), 0);
 #pragma unroll 4
       for (int j = i0 + lane; j < iend; j += 32) {
         const int pay = j < q ? order[j] : 0;
@@ -1044,28 +1127,13 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
         const uint32_t u = u_next + __popc(m & (0xffffffffu >> (31 - lane))) - 1u;
         u_next += __popc(m);
         if (j < q) {
-          write(out0 + j, base + k, pos, bag, u);
+          write_sorted(o, out0 + j, base + k, pos, bag, u);
           // (u < L unless another table's offsets are malformed; then the fallback writes all of this again)
           if (head && (int64_t)u < o.L) put_unique(o, u, base + k, out0 + j);
         }
       }
     }
-    if (r.hot > 0) {
-      const int n = r.seg1 - seg0, first = hot_first ? out0 - r.hot : out0 + q;
-      const uint32_t key = key0 + r.hot_row, u = hot_first ? r.before : r.before + r.mine - 1u;
-      WalkStart start(a, r, n);
-      uint32_t seen = 0;
-      __syncthreads();                                     // everybody is done with what the block kept and with the counters
-      walk_table(a, r, crow, cbag, n, start, r.hot_row, 1u, kNoRow, r.hot, seen,
-                 [&](int, int i, uint32_t, int position, int bag) {
-                   opos[i] = (uint16_t)position;
-                   obag[i] = (uint16_t)bag;
-                 },
-                 [&](int done, int count) {
-                   for (int i = tid; i < count; i += kBsThreads) write(first + done + i, key, seg0 + opos[i], bag0 + obag[i], u);
-                 });
-      if (tid == 0 && (int64_t)u < o.L) put_unique(o, u, key, first);
-    }
+    if (r.hot > 0) copy_row(a, o, r, opos, obag, crow, cbag);
     if (r.id == r.total - 1 && tid == 0) {
       put_segment_end(o, min(r.before + r.mine, (uint32_t)o.L), o.L);
       finish_unique(o, r.before + r.mine);
@@ -1645,9 +1713,9 @@ static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, BucketSort* a, 
   a->T = T; a->B = B; a->N = N;
   a->ranges = T > kBsThreads ? (int)C : 0;
   int bits = 1;
-  while (((uint64_t)(N - 1) >> bits) != 0) ++bits;
+  while (((uint64_t)((N + C - 1) / C - 1) >> bits) != 0) ++bits;   // of a slice of the rows; a longer range takes another pass
   const int passes = (bits + kBsDigit - 1) / kBsDigit;
-  *nb = (bits + passes - 1) / passes;                      // as few passes as a range of all rows takes (most take fewer bits)
+  *nb = (bits + passes - 1) / passes;
   if (*nb < 5) *nb = 5;                                    // the in-block scan wants at least 32 bins
   a->cap = L < kBsCap ? (int)((L + 31) & ~(int64_t)31) : kBsCap;   // small problems leave shared memory to others
   *blocks = a->ranges > 0 ? T * C : T + L / a->per_range;
