@@ -481,10 +481,10 @@ def bench_gpu(args):
     out["kernels"] = kernels
     out["gpu_launches"] = int(round(per_step * cfg.R * K)) + int(round(sum(m["rounds"]) / len(m["rounds"])))
     out["gpu_launches_note"] = "kernel launches of this library inside one timed K-step region (sync on)"
-    out["roofline"] = roofline(kernels, model, host, cfg, peaks)
+    out["roofline"] = roofline(kernels, model, host, cfg, peaks, args.flow_ctas)
     # the same kernel with one replica training alone (no other replica's kernels competing for the SMs)
     k1, _ = profile_pass(model, dev, cfg, replicas=[0])
-    alone = roofline({out["roofline"]["kernel"]: k1[out["roofline"]["kernel"]]}, model, host, cfg, peaks) \
+    alone = roofline({out["roofline"]["kernel"]: k1[out["roofline"]["kernel"]]}, model, host, cfg, peaks, args.flow_ctas) \
         if out["roofline"]["kernel"] in k1 else None
     if alone:
         out["roofline"]["one_replica_alone"] = {k: alone[k] for k in ("achieved", "frac", "us_per_launch")}
@@ -551,7 +551,7 @@ def bench_leg(cfg, K, W, device, args, peaks):
     value, on, info = summarise_training(m, K)
     kernels, per_step = profile_pass(model, dev, cfg, steps=3)
     leg = {"value": value, "unit": UNIT, "ms_per_step": on["median_ms"] / K, "config": {"workload": workload_text(cfg)},
-           "sync": info, "roofline": roofline(kernels, model, host, cfg, peaks),
+           "sync": info, "roofline": roofline(kernels, model, host, cfg, peaks, args.flow_ctas),
            "kernel_launches_per_replica_step": per_step, "status_word": model.status()}
     del graphs, dev, host, model
     return leg
@@ -742,7 +742,7 @@ def profile_pass(model, dev, cfg, steps=6, replicas=None):
     return table, len(recs) / n_rs
 
 
-def roofline(kernels, model, host, cfg, peaks):
+def roofline(kernels, model, host, cfg, peaks, flow_ctas):
     """Roofline entry of the kernel with the largest share of the step's kernel time.
 
     Algorithmic work per launch: embedding forward L(4D+4) + 4(TB+1) + TB*D*{2,4} bytes; fused window kernel
@@ -785,11 +785,9 @@ def roofline(kernels, model, host, cfg, peaks):
         # the launch deliberately takes only some of the SMs (the other replicas' kernels run on the rest), so the
         # fraction of the whole device's peak understates the kernel: give the share of the SMs it holds as well
         import torch
-        from paper_2003_03477_b200 import binding as ss
         sms = torch.cuda.get_device_properties(model.center.device).multi_processor_count
-        ctas = ss.ss_mlp_set_flow_ctas(-1)
-        if ctas == 32:                                       # the library's rule: 192 CTAs shared, 32 to 48 each
-            ctas = max(32, min(48, 192 // cfg.R))
+        # what --flow-ctas set, or the library's rule for several replicas: 192 CTAs shared, 32 to 48 each
+        ctas = flow_ctas if flow_ctas > 0 else (sms if model.sharers == 1 else max(32, min(48, 192 // model.sharers)))
         ctas = min(ctas, sms)
         extra = {"ctas_per_launch": ctas, "sms": sms, "frac_of_the_peak_of_the_sms_it_takes": achieved / peak * sms / ctas,
                  "tensor_pipe_active_pct_ncu": ncu_traffic(name, cfg.name, "tensor_pipe_active_pct")}

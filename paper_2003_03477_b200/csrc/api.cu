@@ -11,7 +11,7 @@ static int g_sms[64];
 
 ss_status check_arch() {
   int dev = 0;
-  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(current_device(&dev));
   if (dev < 0 || dev >= 64) return SS_ERR_ARCH;
   if (g_arch_ok[dev] == 0) {
     int major = 0, sms = 0;
@@ -25,7 +25,7 @@ ss_status check_arch() {
 
 int num_sms() {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if (current_device(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
   if (g_arch_ok[dev] == 0) check_arch();
   return g_sms[dev] > 0 ? g_sms[dev] : 148;
 }

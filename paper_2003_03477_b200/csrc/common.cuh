@@ -25,7 +25,7 @@ inline ss_status cuda_fail(cudaError_t e) {
 // Launch check: picks up a failed launch without synchronising.
 #define SS_LAUNCH_OK()                                  \
   do {                                                  \
-    cudaError_t e__ = cudaGetLastError();               \
+    cudaError_t e__ = ss::g_step_sink ? cudaSuccess : cudaGetLastError(); \
     if (e__ != cudaSuccess) return ss::cuda_fail(e__);  \
   } while (0)
 
@@ -44,11 +44,18 @@ struct StepSink {
   virtual cudaError_t kernel(const LaunchShape& shape, cudaStream_t st, void** params, const size_t* sizes, int n) = 0;
   virtual cudaError_t record(cudaEvent_t e, cudaStream_t st) = 0;
   virtual cudaError_t wait(cudaStream_t st, cudaEvent_t e) = 0;
+  virtual void ctas(int n) = 0;                            // how many CTAs a tensor-core launch was given
+  int device = 0;
  protected:
   ~StepSink() = default;
 };
 extern thread_local StepSink* g_step_sink;
 cudaError_t launch_now(const LaunchShape& shape, cudaStream_t st, void** params);   // a programmatic dependent launch
+inline cudaError_t current_device(int* dev) {              // (a step asks two to four dozen times)
+  if (!g_step_sink) return cudaGetDevice(dev);
+  *dev = g_step_sink->device;
+  return cudaSuccess;
+}
 inline cudaError_t step_record(cudaEvent_t e, cudaStream_t st) { return g_step_sink ? g_step_sink->record(e, st) : cudaEventRecord(e, st); }
 inline cudaError_t step_wait(cudaStream_t st, cudaEvent_t e) { return g_step_sink ? g_step_sink->wait(st, e) : cudaStreamWaitEvent(st, e, 0); }
 

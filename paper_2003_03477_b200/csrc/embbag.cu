@@ -896,7 +896,7 @@ __device__ __forceinline__ void write_sorted(const SortOut& o, int j, uint32_t k
 }
 
 // The range's rows by quantiles of samples: r.base, r.span, r.hot_row, and the rows whose lookups the walk is to count.
-__device__ __noinline__ void recut(const BucketSort& a, BucketRange& r, uint32_t* hist) {
+__device__ __forceinline__ void recut(const BucketSort& a, BucketRange& r, uint32_t* hist) {
   const int tid = threadIdx.x, n = r.seg1 - r.seg0, c = r.c, C = r.ranges;
   uint32_t sample[2];
 #pragma unroll
@@ -918,8 +918,45 @@ __device__ __noinline__ void recut(const BucketSort& a, BucketRange& r, uint32_t
   }
 }
 
-// Outputs of the row of a range that is not sorted.  Out of line: few ranges have one, and inside the kernel its registers
-// cost every range (26 tables of 21 500 lookups 43 -> 45 us).
+// Collects the range's lookups (rows [r.base, r.base + r.span)) in shared memory, as many as fit, and counts those of rows
+// before each of r.edges into r.lt; their number, or -1: the list is malformed.
+__device__ __forceinline__ int collect(const BucketSort& a, BucketRange& r, int n, uint32_t* okey, uint16_t* opos, uint16_t* obag,
+                                       uint32_t* crow, uint16_t* cbag) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cap = a.cap;
+  WalkStart start(a, r, n);
+  __syncthreads();                                         // the range is set
+  const uint32_t base = r.base;
+  const int n_edges = r.n_edges;
+  uint32_t seen[2] = {0u, 0u};
+  const int kept = walk_table(a, r, crow, cbag, n, start, base, r.span, n_edges, seen,
+                              [&](int at, int, uint32_t row, int position, int bag) {
+                                if (at >= cap) return;
+                                okey[at] = row - base;
+                                opos[at] = (uint16_t)position;
+                                obag[at] = (uint16_t)bag;
+                              }, [](int, int) {});
+  for (int j = 0; j < n_edges; ++j) {
+    const uint32_t c = __reduce_add_sync(0xffffffffu, (seen[j >> 2] >> 8 * (j & 3)) & 0xffu);
+    if (lane == 0) r.part[j][warp] = c;
+  }
+  __syncthreads();
+  if (warp < n_edges) {
+    const int c = (int)__reduce_add_sync(0xffffffffu, r.part[warp][lane]);
+    if (lane == 0) r.lt[warp] = c;
+  }
+  __syncthreads();
+  return kept;
+}
+
+// The same once more, by quantiles.  Out of line, like copy_row: few tables need it, and inside the kernel its registers cost
+// every range (26 tables of 21 500 lookups 43 -> 45 us).
+__device__ __noinline__ int collect_again(const BucketSort& a, BucketRange& r, int n, uint32_t* okey, uint16_t* opos, uint16_t* obag,
+                                          uint32_t* crow, uint16_t* cbag) {
+  recut(a, r, okey);
+  return collect(a, r, n, okey, opos, obag, crow, cbag);
+}
+
+// Outputs of the row of a range that is not sorted.
 __device__ __noinline__ void copy_row(const BucketSort& a, const SortOut& o, BucketRange& r, uint16_t* opos, uint16_t* obag,
                                       uint32_t* crow, uint16_t* cbag) {
   const int tid = threadIdx.x, seg0 = r.seg0, n = r.seg1 - seg0, bag0 = r.t * a.B;
@@ -1020,42 +1057,21 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
       __syncthreads();
     }
     // ---- the range's rows, and its lookups into shared memory
-    const bool sound = sound_table(a, o.L, r.t, r.seg0, r.seg1);
-    for (int attempt = 0;; ++attempt) {
+    {
+      const bool sound = sound_table(a, o.L, r.t, r.seg0, r.seg1);
       const int n = sound ? r.seg1 - r.seg0 : 0, C = r.ranges;
-      WalkStart start(a, r, n);
-      if (attempt > 0) {
-        recut(a, r, okey);
-      } else if (tid < kBsMaxBuckets) {
+      if (tid < kBsMaxBuckets) {
         const uint32_t width = ((uint32_t)a.N + C - 1u) / C, edge = min((tid + 1u) * width, (uint32_t)a.N);
         if (tid < kBsMaxBuckets - 1) r.edges[tid] = edge;
         if (tid == r.c) { r.base = min(tid * width, (uint32_t)a.N); r.span = edge - r.base; r.hot_row = kNoRow; r.n_edges = C - 1; }
       }
-      __syncthreads();
-      const uint32_t base = r.base;
-      const int n_edges = r.n_edges;
-      uint32_t seen[2] = {0u, 0u};
-      const int kept = walk_table(a, r, crow, cbag, n, start, base, r.span, n_edges, seen,
-                                  [&](int at, int, uint32_t row, int position, int bag) {
-                                    if (at >= cap) return;
-                                    okey[at] = row - base;
-                                    opos[at] = (uint16_t)position;
-                                    obag[at] = (uint16_t)bag;
-                                  }, [](int, int) {});
-      for (int j = 0; j < n_edges; ++j) {
-        const uint32_t c = __reduce_add_sync(0xffffffffu, (seen[j >> 2] >> 8 * (j & 3)) & 0xffu);
-        if (lane == 0) r.part[j][warp] = c;
-      }
-      __syncthreads();
-      if (warp < n_edges) {
-        const int c = (int)__reduce_add_sync(0xffffffffu, r.part[warp][lane]);
-        if (lane == 0) r.lt[warp] = c;
-      }
-      __syncthreads();
-      int fullest = kept;                                  // of the range, or of all slices of the table
-      if (attempt == 0) {
-        for (int c = 0; c < C; ++c) fullest = max(fullest, (c < C - 1 ? r.lt[c] : n) - (c > 0 ? r.lt[c - 1] : 0));
-        if (kept >= 0 && C > 1 && fullest > cap) continue;
+      int kept = collect(a, r, n, okey, opos, obag, crow, cbag);
+      int fullest = kept, before = r.c > 0 ? r.lt[r.c - 1] : 0, hot = 0;
+      for (int c = 0; c < C; ++c) fullest = max(fullest, (c < C - 1 ? r.lt[c] : n) - (c > 0 ? r.lt[c - 1] : 0));   // of all slices
+      if (kept >= 0 && C > 1 && fullest > cap) {
+        fullest = kept = collect_again(a, r, n, okey, opos, obag, crow, cbag);
+        before = r.lt[0];
+        hot = r.hot_row == kNoRow ? 0 : r.lt[2] - r.lt[1];
       }
       const bool ok = sound && kept >= 0 && fullest <= cap;
       const int q = ok ? kept : 0;
@@ -1064,11 +1080,10 @@ bucket_sort_kernel(const __grid_constant__ BucketSort a, const __grid_constant__
       if (tid == 0) {
         if (!ok) atomicOr(a.fallback, 1);
         r.kept = q;
-        r.hot = ok && n_edges == 3 && attempt > 0 ? r.lt[2] - r.lt[1] : 0;
-        r.out0 = r.seg0 + (attempt > 0 ? r.lt[0] : (r.c > 0 ? r.lt[r.c - 1] : 0));
+        r.hot = ok ? hot : 0;
+        r.out0 = r.seg0 + before;
       }
       __syncthreads();
-      break;
     }
     // ---- sort
     const int q = r.kept, q32 = (q + 31) & ~31;
@@ -1257,7 +1272,7 @@ window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restric
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // ---- (4b) fused window kernel for rows of at most 4G floats ------------------------------------
-// Same windows, same order of additions and same outputs as window_reduce_kernel<G, 1, true>.  The run
+// Same windows and same order of additions as window_reduce_kernel.  The run
 // structure of the window is three 16-bit masks (valid, head, tail) built once from the keys; while the
 // keys are looked at, the table rows of the window's runs are requested into L2, so that when a run ends
 // its row is updated on the spot from the sum in the lanes' registers.  No shared-memory stash: the number
@@ -1631,7 +1646,7 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
 }
 
 template <int G, int NV>
-static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, const int32_t* perm, int T, int64_t N,
+static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
                           int D, int B, const float* grad, int64_t ld_grad, int col0, float* tables,
                           float* row_state, float lr, float eps, int32_t* d_status, cudaStream_t st) {
   constexpr int kGroups = 256 / G;
@@ -1726,7 +1741,7 @@ template <int NB>
 static ss_status launch_bucket_sort_nb(const BucketSort& a, const TiledSort& t, int64_t blocks, cudaStream_t st) {
   static bool attr_set[64];
   int dev = 0;
-  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(current_device(&dev));
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     SS_CUDA(cudaFuncSetAttribute(bucket_sort_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs_smem(kBsCap, NB)));
     attr_set[dev] = true;
@@ -1863,7 +1878,7 @@ static ss_status bwd_impl(bool do_sort, bool do_apply, float* tables, float* row
   // (4) windowed segment reduction, (5) combine, (6) row-wise Adagrad
   if (do_apply) {
 #define SS_RED(G_, NV_) \
-  launch_reduce<G_, NV_>(p, ws, keys_sorted, perm_sorted, T, N, D, B, grad, ld_grad, col0, tables, row_state, lr, eps, d_status, cs)
+  launch_reduce<G_, NV_>(p, ws, keys_sorted, T, N, D, B, grad, ld_grad, col0, tables, row_state, lr, eps, d_status, cs)
     SS_DISPATCH_GNV(D, SS_RED);
 #undef SS_RED
     SS_LAUNCH_OK();
@@ -1913,7 +1928,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 static ss_status noalloc_scratch_ptr(unsigned char** out) {
   static unsigned char* ptr[64];
   int dev = 0;
-  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(ss::current_device(&dev));
   if (dev < 0 || dev >= 64) return SS_ERR_SHAPE;
   if (!ptr[dev]) {
     void* p = nullptr;

@@ -94,6 +94,8 @@ ss_status gemm_tc_flow(const TcJob* jobs, int n, int* ctrl, int max_rows, int sh
 // CTAs a flow with dependencies takes (0: by the library's rule, negative: no change); returns the number set, or the
 // least the rule gives.
 int set_flow_ctas(int ctas);
+// How many CTAs the rule gives a flow launched into `st` now (and takes note of that launch).
+int flow_ctas(int sharers, cudaStream_t st);
 // The device error flag raised by a bounded wait that ran out (0 = none); synchronises the device.
 int read_device_error(bool clear);
 

@@ -208,7 +208,7 @@ static ss_status launch_f32(F32Jobs& jobs, int blocks, cudaStream_t st) {
   constexpr size_t smem = (size_t)kFStages * (BM + BN) * kFRow * 4;
   static bool attr_set[64];
   int dev = 0;
-  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(current_device(&dev));
   if (smem > 48 * 1024 && dev >= 0 && dev < 64 && !attr_set[dev]) {
     SS_CUDA(cudaFuncSetAttribute(gemm_f32_kernel<BM, BN, TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_set[dev] = true;

@@ -876,7 +876,7 @@ static bool make_map_atoms(CUtensorMap* map, const void* base, int64_t rows, int
 static int* device_error_ptr() {
   static int* ptr[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  if (current_device(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   if (!ptr[dev]) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_device_error) != cudaSuccess) return nullptr;
@@ -908,7 +908,7 @@ template <int kStages, int kBN, int kBK, bool kPair>
 static ss_status launch_flow(const TcFlow<kTcMaxFlow>& f, int ctas, cudaStream_t st) {
   static bool attr_set[64];
   int dev = 0;
-  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(current_device(&dev));
   const size_t smem = tc_smem_bytes(kStages, kPair ? kBN / 2 : kBN, kBK, sizeof(TcMeta) * kTcMaxFlow);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     SS_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<kStages, kBN, kBK, kTcMaxFlow, kPair>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1007,14 +1007,14 @@ int set_flow_ctas(int ctas) {
   return g_flow_ctas > 0 ? g_flow_ctas : kFlowCtasMin;
 }
 
-static int flow_ctas(int sharers, cudaStream_t st) {
+int flow_ctas(int sharers, cudaStream_t st) {
   constexpr int kRecent = 8;
   struct Recent { cudaStream_t stream[kRecent]; unsigned next, filled; };
   static Recent recent[64];
   static std::mutex lock;
   if (g_flow_ctas > 0) return g_flow_ctas;
   int dev = 0, streams = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+  if (current_device(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
     std::lock_guard<std::mutex> guard(lock);
     Recent& r = recent[dev];
     r.stream[r.next++ % kRecent] = st;
@@ -1037,6 +1037,7 @@ static int flow_ctas(int sharers, cudaStream_t st) {
 // (12 KiB each) for the process, looked up by all of their arguments.
 static ss_status build_flow(const TcJob* jobs, int n, int* ctrl, int max_rows, int bn, int bk, bool pair, int* err, TcFlow<kTcMaxFlow>* out) {
   TcFlow<kTcMaxFlow>& f = *out;
+  memset(out, 0, sizeof(*out));                            // padding too: launches are compared byte by byte (step.cu)
   f.n = n;
   int total = 0;
   for (int i = 0; i < n; ++i) {
@@ -1120,6 +1121,7 @@ ss_status gemm_tc_flow(const TcJob* jobs, int n, int* ctrl, int max_rows, int sh
   int ctas = num_sms();
   if (ctrl) {
     const int share = flow_ctas(sharers, st);
+    if (g_step_sink) g_step_sink->ctas(share);
     if (share < ctas) ctas = share;
   }
   // Tile width.  128 x 256 tiles where the flow has three of them for two CTAs; with fewer, a layer takes as long as the k
@@ -1139,7 +1141,6 @@ ss_status gemm_tc_flow(const TcJob* jobs, int n, int* ctrl, int max_rows, int sh
   const bool pair = wide && ctas >= 2 && (ctrl ? t_pair >= 2 * ctas && kb_pair >= 12 * t_pair : t_pair >= ctas / 2);
   const int bn = wide ? 256 : 64;
   alignas(64) TcFlow<kTcMaxFlow> f;
-  memset(&f, 0, sizeof(f));                                // padding too: launches are compared byte by byte (step.cu)
   ss_status built;
   try {
     built = flow_plan(jobs, n, ctrl, max_rows, bn, pair, err, &f);

@@ -5,6 +5,7 @@
 // route pays a Python call per attribute: the host side of a small call is mostly this.  Nothing is computed here.
 #include <torch/csrc/autograd/python_variable.h>
 #include <c10/cuda/CUDAStream.h>
+#include <string.h>
 #include "../../include/shadowsync.h"
 
 namespace {
@@ -277,6 +278,7 @@ SS_PY(sync_bmuf) {
 SS_PY(train_step) {
   return guarded(args, nargs, [](Args& a) {
     ss_step_args s;
+    memset(&s, 0, sizeof(s));       // padding too: a plan compares steps byte by byte
     s.desc = a.desc();
     s.tables = a.ptr<float>(); s.row_state = a.ptr<float>();
     s.T = a.i32(); s.N = a.i64(); s.D = a.i32(); s.B = a.i32();

@@ -109,8 +109,8 @@ def test_medium_workload_first_step_full_size_as_benchmarked():
 
 def test_large_workload_embedding_path_full_size():
     """The embedding calls of the large workload at its full size (26 tables of 4 M rows x 128 floats = 53 GB filled
-    on the device, batch 4096, about 852 k lookups with 27-bit keys): more lookups than the per-table shared-memory
-    sort can hold, so the tiled radix passes run (three digits, about 208 tiles), the hottest row of a table has
+    on the device, batch 4096, about 852 k lookups with 27-bit keys): several ranges a table in the shared-memory sort, the
+    hottest row of a table has
     thousands of lookups (runs spanning hundreds of reduction windows) and rows are 128 floats wide.  Forward, sort
     (integers bit-exact) and reduction + row-wise Adagrad against the oracle on the compact table of touched rows;
     the gradient is a seeded synthetic matrix, so no MLP (and no ReLU gate) is involved."""
@@ -118,7 +118,7 @@ def test_large_workload_embedding_path_full_size():
     T, N, D, B = cfg.T, cfg.N, cfg.D, cfg.B
     batch = synth.make_batch(cfg, 0, 0)
     L = batch.L
-    assert L > T * ss.SS_TABLE_SORT_CAP                      # the tiled passes are certain
+    assert L > T * ss.SS_TABLE_SORT_CAP                      # three ranges a table
     tables_c, small, uniq, t_of, local, nmax = _compact(cfg, batch)
     tables = trainer.device_tables(cfg)
     state = torch.zeros(T * N, dtype=torch.float32, device="cuda")
@@ -166,8 +166,8 @@ def test_large_workload_embedding_path_full_size():
 
 
 def test_sort_with_one_table_beyond_the_shared_memory_sort_beside_tables_within_it():
-    """Three tables in one call: the middle one has more lookups than one block of the per-table sort holds
-    (its block raises the fallback word and the tiled passes redo the whole call), the outer two would fit."""
+    """Three tables in one call: the middle one has more lookups than a block of the shared-memory sort holds (it gets more
+    ranges), the outer two would fit into one."""
     T, N, B = 3, 1 << 20, 4096
     rng = np.random.default_rng(11)
     lens = np.concatenate([rng.integers(1, 4, B), rng.integers(6, 12, B), rng.integers(0, 3, B)])
