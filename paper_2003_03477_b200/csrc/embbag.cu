@@ -621,7 +621,10 @@ tiled_sort_kernel(const __grid_constant__ TiledSort a) {
 // which they all read alike.  A popular row on an edge goes to the side that has less of it; where a range is too full all
 // the same, because its first or last row draws so much, that row is not sorted but copied out, in order, by one more walk
 // over the index list.  (Quantiles in the first place, or samples that tell whether slices will do, cost 2-4 us a call.)
-// What bounds it is instruction issue and the latency of a block's rounds.
+// What bounds it is instruction issue and the latency of a block's rounds.  Measured alone, the whole sort half, ids scattered /
+// ordered by popularity / one row drawing 80 % (in brackets slices with a fixed reserve for a popular row, and the tiled
+// passes behind them where those overflowed): 26 tables of 21 500 lookups 44 / 60 / 67 us (43 / 152 / 147), 26 of 32 800
+// 58 / 77 / 103 (49 / 164 / 161), 40 of 32 900 56 / 85 / 115 (74 / 272 / 258).
 //
 // A block that cannot take the path (a range with more lookups than `cap` after all, a table of more than 65536, offsets
 // that are not monotone within [0, L], a row index outside the table) raises *fallback.  Only a range can be too full if
@@ -1711,8 +1714,9 @@ __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_f
 
 // Whether the bucket sort takes a problem, how many lookups it gives a range, and the most ranges there can be, whatever the
 // tables' lengths: a block for each.  Every further range reads the index list once more and holds an SM, so a table gets as
-// few ranges as hold its lookups.  Few tables are cut finer, down to 5500 lookups a range, while that takes no more than a
-// quarter of the SMs (5 tables of 9000 lookups: 91 -> 79 us for lookup and update).
+// few ranges as hold its lookups (four replicas of the ordinary model 478 us a round with two ranges a table, 494 with three).
+// Few tables are cut finer, down to 5500 lookups a range, while that takes no more than a quarter of the SMs (5 tables of
+// 9000 lookups: 91 -> 79 us for lookup and update).  Blocks without a range cost nothing that could be measured.
 static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, BucketSort* a, int64_t* blocks, int* nb) {
   const int64_t avg = (L + T - 1) / T;
   if (B > 65535 || avg > 44000) return false;              // bag numbers, plus one, take 16 bits

@@ -100,7 +100,7 @@ class Replica:
         # and the embedding calls a level in between (still above the shadow stream): blocks of an MLP kernel
         # are placed as soon as a slot frees up instead of queueing behind another replica's gather.
         self.stream = torch.cuda.Stream(device=dev, priority=model.prio_embedding)
-        # the index sort of the backward runs here: one block per table on few SMs, and the reduction waits for it,
+        # the index sort of the backward runs here: a few blocks per table, and the reduction waits for it,
         # so it goes in between where the device has a level left (measured +2 % examples/s)
         self.side = torch.cuda.Stream(device=dev, priority=model.prio_sort)
         self.mlp = torch.cuda.Stream(device=dev, priority=priority)
@@ -129,10 +129,10 @@ class Model:
         lo, hi = torch.cuda.Stream.priority_range()   # (lowest priority value, highest), e.g. (0, -5)
         self.prio_low, self.prio_high = lo, hi
         self.prio_embedding = hi + min(2, max(0, (lo - hi) - 1))   # between the two when the device has the levels
-        # only while the sort is the light per-table kernel: the tiled passes of larger batches fill the device and,
-        # given precedence over the other replicas' embedding calls, cost a quarter of the throughput (measured)
-        # ... and while the sorts of all replicas together (one SM per table each) leave SMs free: with R*T beyond the
-        # SM count the raised level costs 2 % instead of gaining 2 % (measured at R=8, T=26)
+        # only while the sort takes few SMs (at most two blocks a table): the tiled passes of the longest tables fill the
+        # device and, given precedence over the other replicas' embedding calls, cost a quarter of the throughput (measured)
+        # ... and not with many replicas and tables: with R*T beyond the SM count the raised level cost 2 % (R=8, T=26);
+        # below it, it gains 2 % (a round of R=4, T=26, two blocks a table: 480 us, 490 on the embedding calls' level)
         light_sort = 0 < max_L <= T * ss.SS_TABLE_SORT_CAP and R * workers * T <= ss.ss_num_sms()
         self.prio_sort = self.prio_embedding - 1 if (light_sort and self.prio_embedding - 1 > hi) else self.prio_embedding
         self.replicas: List[Replica] = [Replica(self, w0_flat, hi, max_L, keep_sort_outputs) for _ in range(R)]
