@@ -1274,16 +1274,88 @@ window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restric
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// ---- (4b) fused window kernel for rows of at most 4G floats ------------------------------------
-// Same windows and same order of additions as window_reduce_kernel.  The run
-// structure of the window is three 16-bit masks (valid, head, tail) built once from the keys; while the
-// keys are looked at, the table rows of the window's runs are requested into L2, so that when a run ends
-// its row is updated on the spot from the sum in the lanes' registers.  No shared-memory stash: the number
-// of windows in flight on an SM is bounded by registers only.
+// ---- (4b) fused window kernel for rows of at most 128 floats --------------------------------------
+// Same windows and same order of additions as window_reduce_kernel.  A block stages keys and gradient rows of its windows
+// together (32 consecutive positions per warp and round) and requests the table rows of the runs into L2; ballots give the run
+// structure of a window as 16-bit masks.  A batch of positions requests its gradient rows and, for the runs that end in it, the
+// table rows and states at once; then it adds, and updates a row where a run ends.  A run of up to kShortSpan windows of one
+// block is finished by the group it starts in, so only runs that leave the block, and long ones, are left to the combine kernel.
+// What bounds it is latency and instruction issue together (half of the issue slots, 45 % of the warp slots): rows one after
+// the other as their runs end, and a thread's keys by itself, took 46 us for 26 skewed tables of 21 500 lookups of 64 floats
+// (with the combine kernel 58; now 42 and 51), 100 us for 40 tables of 32 900 of 16 floats (now 84), 16 for 11 of 10 700 of
+// 48 (the same; with the combine kernel 21, now 19).  Additions and steps take two floats an instruction.
+constexpr int kShortSpan = 8;                              // most windows whose parts one lane group adds
 constexpr int kWaThreads = 128;
 
+// 16 bytes of a row: two packed pairs of floats.  Pairs are added and multiplied two floats an instruction, each rounded as by
+// itself.
+struct Quad { uint64_t a, b; };
+__device__ __forceinline__ uint64_t add_pair(uint64_t x, uint64_t y) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma_pair(uint64_t x, uint64_t y, uint64_t z) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+  return d;
+}
+__device__ __forceinline__ Quad add_quad(Quad x, Quad y) { return Quad{add_pair(x.a, y.a), add_pair(x.b, y.b)}; }
+__device__ __forceinline__ float4 floats_of(Quad q) {
+  return make_float4(__uint_as_float((uint32_t)q.a), __uint_as_float((uint32_t)(q.a >> 32)), __uint_as_float((uint32_t)q.b),
+                     __uint_as_float((uint32_t)(q.b >> 32)));
+}
+__device__ __forceinline__ Quad quad_nc(const char* p) {
+  const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
+  return Quad{v.x, v.y};
+}
+__device__ __forceinline__ Quad quad_at(const char* p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  return Quad{v.x, v.y};
+}
+
+// The columns of a lane in a group of G, NV float4 each G float4 apart: byte offsets inside a row.  Exact: the row is
+// G * NV float4 wide.  Otherwise a lane whose column lies beyond the row reads another one in its place and stores nothing.
+template <int G, int NV, bool Exact>
+struct LaneColumns {
+  int nvec, lane;
+  __device__ __forceinline__ LaneColumns(int nvec_, int lane_) : nvec(nvec_), lane(lane_) {}
+  __device__ __forceinline__ bool inside(int v) const { return Exact || lane + v * G < nvec; }
+  __device__ __forceinline__ uint32_t first() const { return 16u * (uint32_t)(Exact || lane < nvec ? lane : 0); }
+  __device__ __forceinline__ uint32_t next(int v) const { return inside(v) ? 16u * v * G : 0u; }   // beyond first()
+};
+
+// Sum over the group of g^2, the same in every lane.  The lanes' parts are added in the order of a tree over 2 * G lanes (H = 2)
+// or G lanes (H = 1): with H = 2 a lane holds what two lanes G apart would hold.
+template <int G, int NV, int H>
+__device__ __forceinline__ float square_sum(const float4 (&g)[NV], unsigned mask) {
+  float part[H];
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    part[h] = 0.f;
+#pragma unroll
+    for (int v = h; v < NV; v += H)
+      part[h] += __fmaf_rn(g[v].w, g[v].w, __fmaf_rn(g[v].z, g[v].z, __fmaf_rn(g[v].x, g[v].x, __fmul_rn(g[v].y, g[v].y))));
+  }
+  float ss = H == 2 ? part[0] + part[H - 1] : part[0];
+#pragma unroll
+  for (int off = G / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(mask, ss, off, G);
+  return ss;
+}
+
+// The row's new state and the factor of its gradient.  Wide: rows of more than 128 floats, whose quotients are rounded exactly;
+// for the others the reciprocal of D is loop-invariant and the quotient is within 2 ulp.
+template <bool Wide>
+__device__ __forceinline__ float next_state(float st, float ss, int D) {
+  return Wide ? st + ss / (float)D : __fmaf_rn(ss, 1.0f / (float)D, st);
+}
+template <bool Wide>
+__device__ __forceinline__ float step_scale(float lr, float sn, float eps) {
+  return Wide ? lr / (sqrtf(sn) + eps) : __fdividef(lr, sqrtf(sn) + eps);
+}
+
 // Row-wise Adagrad on one row whose gradient is in the lanes' registers, NV float4 per lane (column lane + v*G).
-template <int G, int NV>
+template <int G, int NV, bool Wide>
 __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t key, int lane, int nvec, int D,
                                                unsigned gmask, float* __restrict__ tables,
                                                float* __restrict__ row_state, float lr, float eps) {
@@ -1292,14 +1364,8 @@ __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t k
 #pragma unroll
   for (int v = 0; v < NV; ++v) r[v] = (lane + v * G < nvec) ? row[lane + v * G] : make_float4(0.f, 0.f, 0.f, 0.f);
   const float st = row_state[key];
-  float ss = 0.f;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) ss += g[v].x * g[v].x + g[v].y * g[v].y + g[v].z * g[v].z + g[v].w * g[v].w;
-#pragma unroll
-  for (int off = G / 2; off >= 1; off >>= 1) ss += __shfl_down_sync(gmask, ss, off, G);
-  ss = __shfl_sync(gmask, ss, 0, G);                       // every lane uses lane 0's sum
-  const float sn = st + ss * (1.0f / (float)D);            // the reciprocal is loop-invariant at the call sites
-  const float scale = __fdividef(lr, sqrtf(sn) + eps);     // within 2 ulp of the quotient
+  const float ss = square_sum<G, NV, 1>(g, gmask);
+  const float sn = next_state<Wide>(st, ss, D), scale = step_scale<Wide>(lr, sn, eps);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     if (lane + v * G < nvec) {
@@ -1312,118 +1378,202 @@ __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t k
   if (lane == 0) row_state[key] = sn;
 }
 
-template <int G, int NV>
-__global__ void __launch_bounds__(kWaThreads, 8)
+template <int G, int NV, int H, int KB, int kMinBlocks, bool Exact, bool Wide>
+__global__ void __launch_bounds__(kWaThreads, kMinBlocks)
 window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
-                    const int32_t* __restrict__ uidx, int64_t L, uint32_t sentinel, int64_t N, int D, int B,
+                    const int32_t* __restrict__ uidx, int L, uint32_t sentinel, int T, uint32_t N, int D, int B,
                     const float* __restrict__ grad, int64_t ld_grad, int col0, float* __restrict__ partial,
-                    int32_t* __restrict__ long_list, int32_t* __restrict__ scalars, int nwin, int64_t umax,
+                    int32_t* __restrict__ long_list, int32_t* __restrict__ scalars, int nwin,
                     int32_t* __restrict__ d_status, float* __restrict__ tables, float* __restrict__ row_state,
                     float lr, float eps) {
   wait_for_previous_kernel();
-  constexpr int kGroups = kWaThreads / G;
-  __shared__ uint32_t s_key[kGroups][kWin + 2];            // [0] = key before the window, [kWin+1] = key after
-  __shared__ int32_t s_row[kGroups][kWin];                 // float4 index of the lookup's gradient row
-  __shared__ int32_t s_u[kGroups][kWin];
+  constexpr int kGroups = kWaThreads / G, kPos = kGroups * kWin;
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ __align__(16) uint32_t s_key[kPos];
+  __shared__ __align__(16) int32_t s_row[kPos];            // float4 index of the lookup's gradient row
+  __shared__ uint32_t s_valid[kPos / 32], s_head[kPos / 32];
+  static_assert(kPos % 32 == 0, "whole warps stage positions");
   const int grp = threadIdx.x / G, lane = threadIdx.x % G;
-  const int64_t win = (int64_t)blockIdx.x * kGroups + grp;
-  const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) / G * G));
   if (!ws_matches(scalars, L, sentinel, d_status)) return;
-  if (win >= nwin) return;
-  const int64_t w0 = win * kWin;
-  const int nvec = D >> 2;
-  const int64_t ld4 = ld_grad >> 2;
-  for (int e = lane; e < kWin + 2; e += G) {
-    const int64_t j = w0 - 1 + e;
-    const bool in_range = j >= 0 && j < L;
-    const bool body = e >= 1 && e <= kWin;
-    uint32_t key = in_range ? keys[j] : sentinel;
-    const int sb = (body && in_range) ? sbag[j] : 0;
-    const int u = (body && in_range) ? uidx[j] : 0;
-    int32_t row = -1;
-    if (body && key < sentinel) {
-      const int t = (int)((uint32_t)sb / (uint32_t)B);     // bags are table-major: bag = t*B + b
-      const int b = sb - t * B;
-      // a consistent workspace never fails these; an inconsistent one must not turn into a wild access
-      if (sb >= 0 && (int64_t)key >= (int64_t)t * N && (int64_t)key < (int64_t)(t + 1) * N && u >= 0 && u < umax) {
-        row = (int32_t)((int64_t)b * ld4 + (int64_t)t * nvec);   // B * ld_grad / 4 < 2^31 is checked on the host
-        const char* trow = reinterpret_cast<const char*>(tables + (int64_t)key * D);
-        for (int o = 0; o < D * 4; o += 128) prefetch_l2(trow + o);     // a repeated key asks for a line already on its way
-        prefetch_l2(row_state + key);
-      } else {
-        key = sentinel;
+  const LaneColumns<G, NV, Exact> col(D >> 2, lane);
+  const uint32_t row_bytes = (uint32_t)D * 4u;
+  const int p0 = (int)blockIdx.x * kPos;                   // the block's first position (below L < 2^31)
+  // ---- keys, gradient rows and run structure of the block's positions, 32 consecutive ones per warp and round
+  {
+    const int nvec = D >> 2, ld4 = (int)(ld_grad >> 2);    // B * ld_grad / 4 < 2^31 is checked on the host
+    int t = (int)((uint32_t)sbag[p0] / (uint32_t)B);       // table of the block's first position
+#pragma unroll
+    for (int e0 = 0; e0 < kPos; e0 += kWaThreads) {
+      const int e = e0 + threadIdx.x, j = p0 + e;
+      if (kPos % kWaThreads != 0 && e >= kPos) break;      // (whole warps)
+      uint32_t key = sentinel, before = sentinel;
+      int32_t row = -1;
+      if (j < L) {
+        key = keys[j];
+        const int sb = sbag[j];
+        if (j > 0) before = keys[j - 1];
+        if (key < sentinel) {
+          int b = sb - t * B;                              // bags are table-major: bag = t*B + b
+          if ((uint32_t)b >= (uint32_t)B) { t = (int)((uint32_t)sb / (uint32_t)B); b = sb - t * B; }
+          // a consistent workspace never fails these; an inconsistent one must not turn into a wild access
+          if (sb >= 0 && t < T && key - (uint32_t)t * N < N) row = b * ld4 + t * nvec;
+          else key = sentinel;
+        }
       }
-    }
-    s_key[grp][e] = key;
-    if (body) { s_row[grp][e - 1] = row; s_u[grp][e - 1] = u; }
-  }
-  __syncwarp(gmask);
-  // valid (bits 16..31) and head (bits 0..15) of the positions this lane owns, then OR over the group
-  uint32_t bits = 0;
-  for (int i = lane; i < kWin; i += G) {
-    const uint32_t k = s_key[grp][1 + i];
-    if (k < sentinel) {
-      bits |= 0x10000u << i;
-      if (i == 0 || s_key[grp][i] != k) bits |= 1u << i;
-    }
-  }
+      const bool valid = row >= 0, head = valid && (before != key || (e & (kWin - 1)) == 0);
+      if (head) {                                          // request the run's row into L2
+        const char* trow = reinterpret_cast<const char*>(tables) + (uint64_t)key * row_bytes;
+        if (Exact) {
 #pragma unroll
-  for (int off = G / 2; off >= 1; off >>= 1) bits |= __shfl_xor_sync(gmask, bits, off, G);
-  const uint32_t vm = bits >> 16, hm = bits & 0xffffu;
-  // a run ends where the next position starts another run, is a skipped lookup, or lies outside the window
-  const uint32_t tm = vm & ((hm >> 1) | (~vm >> 1) | 0x8000u);
-  const bool first_open = (vm & 1u) && s_key[grp][0] == s_key[grp][1];
-  const bool last_open = (vm >> (kWin - 1) & 1u) && s_key[grp][kWin + 1] == s_key[grp][kWin];
-  const float4* grad4 = reinterpret_cast<const float4*>(grad + col0);  // col0 is a multiple of 4
-
-  float4 acc[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-  constexpr int kBatch = 8 / NV;                           // gradient rows in flight per lane (8 float4)
-  // (rolled for 128-wide rows: 84 -> 74 us on 26 skewed tables of 33 400 lookups; narrower rows are faster unrolled, 47 us against 49)
-  constexpr int kUnroll = G >= 16 ? 1 : kWin / kBatch;
-#pragma unroll kUnroll
-  for (int i0 = 0; i0 < kWin; i0 += kBatch) {
-    float4 gv[kBatch][NV];
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int32_t row = s_row[grp][i0 + u];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const int c = lane + v * G;
-        gv[u][v] = (row >= 0 && c < nvec) ? __ldg(grad4 + row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int i = i0 + u;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        if ((hm >> i) & 1u) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[v] = add4(acc[v], gv[u][v]);                   // skipped lookups carry zeros and follow every run
-      }
-      if ((tm >> i) & 1u) {
-        const uint32_t key = s_key[grp][1 + i];
-        const bool first = (tm & ((1u << i) - 1u)) == 0u;  // the window's first run holds position 0
-        const bool head_open = first && first_open;
-        const bool tail_open = (i == kWin - 1) && last_open;
-        if (!head_open && !tail_open) {
-          adagrad_row_nv<G, NV>(acc, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
+          for (int o = 0; o < G * NV * 16; o += 128) prefetch_l2(trow + o);
         } else {
+          for (uint32_t o = 0; o < row_bytes; o += 128) prefetch_l2(trow + o);
+        }
+        prefetch_l2(row_state + key);
+      }
+      s_key[e] = key;
+      s_row[e] = max(row, 0);                              // skipped lookups follow every run: what is added for them goes nowhere
+      const uint32_t vb = __ballot_sync(kAll, valid), hb = __ballot_sync(kAll, head);
+      if ((threadIdx.x & 31) == 0) { s_valid[e >> 5] = vb; s_head[e >> 5] = hb; }
+    }
+  }
+  __syncthreads();
+  const int w0 = grp * kWin, win = p0 / kWin + grp;        // the group's window: first position inside the block, number
+  const uint32_t vm = (s_valid[w0 >> 5] >> (w0 & 16)) & 0xffffu, hm = (s_head[w0 >> 5] >> (w0 & 16)) & 0xffffu;
+  // a run ends where the next position starts another run, is a skipped lookup, or lies outside the window
+  const uint32_t tm = vm & ((hm >> 1) | (~vm >> 1) | 0x8000u), first_tail = tm & (0u - tm);
+  bool first_open = false, last_open = false;              // the first / last run goes on in a neighbouring window
+  if (vm & 1u) first_open = p0 + w0 > 0 && (w0 > 0 ? s_key[w0 - 1] : keys[p0 - 1]) == s_key[w0];
+  if (vm >> (kWin - 1)) {
+    const int j = p0 + w0 + kWin;
+    last_open = j < L && (w0 + kWin < kPos ? s_key[w0 + kWin] : keys[j]) == s_key[w0 + kWin - 1];
+  }
+  // runs that end here and are complete; the others leave a partial sum
+  const uint32_t um = tm & ~(first_open ? first_tail : 0u) & ~(last_open ? 0x8000u : 0u);
+  const char* const gl = reinterpret_cast<const char*>(grad + col0) + col.first();   // col0 is a multiple of 4
+  char* const tl = reinterpret_cast<char*>(tables) + col.first();
+  float* const pl = partial + (int64_t)win * 2 * D + (col.first() >> 2);
+
+  // a row's step from the sum of its gradients
+  auto step = [&](const Quad (&g)[NV], const Quad (&r)[NV], float st, uint32_t key, bool store) {
+    float4 f[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) f[v] = col.inside(v) ? floats_of(g[v]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float ss = square_sum<G, NV, H>(f, kAll);
+    const float sn = next_state<Wide>(st, ss, D), scale = -step_scale<Wide>(lr, sn, eps);
+    const uint64_t s2 = (uint64_t)__float_as_uint(scale) << 32 | __float_as_uint(scale);
+    __syncwarp();                                          // every lane has read the state
+    if (store) {
+      char* const p = tl + (uint64_t)key * row_bytes;
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        if (col.inside(v))
+          *reinterpret_cast<ulonglong2*>(p + 16 * v * G) = make_ulonglong2(fma_pair(s2, g[v].a, r[v].a), fma_pair(s2, g[v].b, r[v].b));
+      if (lane == 0) row_state[key] = sn;
+    }
+  };
+
+  Quad acc[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = Quad{0ull, 0ull};
+#pragma unroll 1
+  for (int i0 = 0; i0 < kWin; i0 += KB) {
+    Quad gv[KB][NV], rv[KB][NV];
+    float st[KB];
+    uint32_t key[KB];
+    const uint32_t tails = tm >> i0, upds = um >> i0;
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+      const char* const p = gl + (int64_t)s_row[w0 + i0 + u] * 16;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) gv[u][v] = quad_nc(p + col.next(v));
+    }
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+      key[u] = s_key[w0 + i0 + u];
+      st[u] = 0.f;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) rv[u][v] = Quad{0ull, 0ull};
+      if ((upds >> u) & 1u) {
+        const char* const p = tl + (uint64_t)key[u] * row_bytes;
+        st[u] = row_state[key[u]];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) rv[u][v] = quad_at(p + col.next(v));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = add_quad(acc[v], gv[u][v]);
+      const bool tail = (tails >> u) & 1u, upd = (upds >> u) & 1u;
+      if (__any_sync(kAll, tail)) {
+        step(acc, rv[u], st[u], key[u], upd);
+        if (tail && !upd) {
           // the run goes on in a neighbouring window: its part goes to the window's partial slot
-          // (slot 0 when the run holds the window's first position), the combine kernel adds the parts
-          float4* dst = reinterpret_cast<float4*>(partial + ((int64_t)win * 2 + (first ? 0 : 1)) * D);
+          // (slot 0 when the run holds the window's first position)
+          float* const dst = pl + ((first_tail >> (i0 + u)) & 1u ? 0 : D);
 #pragma unroll
           for (int v = 0; v < NV; ++v)
-            if (lane + v * G < nvec) dst[lane + v * G] = acc[v];
-          if (!head_open && lane == 0) {                   // the window in which a multi-window run starts lists the row
-            const int slot = atomicAdd(&scalars[1], 1);
-            if (slot < nwin) long_list[slot] = s_u[grp][i];   // at most one such run per window
-          }
+            if (col.inside(v)) *reinterpret_cast<ulonglong2*>(dst + 4 * v * G) = make_ulonglong2(acc[v].a, acc[v].b);
+        }
+        if (tail) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc[v] = Quad{0ull, 0ull};
         }
       }
     }
   }
+  // ---- a run that starts in this window and goes on: its parts are added here, in window order, if they are all of this
+  // block and no more than kShortSpan; otherwise the row enters the combine kernel's list
+  __syncthreads();                                         // the block's parts are in memory
+  const bool starts = last_open && !(first_open && first_tail == 0x8000u);
+  const uint32_t key = s_key[w0 + kWin - 1];
+  int span = 0;                                            // windows the run covers, 0: too many or not all of them here
+  if (starts) {
+    int e = grp + 1;
+    while (e < kGroups && e - grp < kShortSpan - 1 && s_key[e * kWin + kWin - 1] == key &&
+           (e + 1 == kGroups || s_key[e * kWin + kWin] == key)) ++e;
+    bool ends = e < kGroups;
+    if (ends && s_key[e * kWin + kWin - 1] == key) {       // up to the window's end: does the next one begin with another row?
+      const int j = p0 + (e + 1) * kWin;
+      ends = j >= L || (e + 1 < kGroups ? s_key[e * kWin + kWin] : keys[j]) != key;
+    }
+    if (ends) {
+      span = e - grp + 1;
+    } else if (lane == 0) {
+      const int u_at = uidx[p0 + w0 + kWin - 1];
+      const int slot = atomicAdd(&scalars[1], 1);
+      if (slot < nwin) long_list[slot] = u_at;             // at most one such run per window
+    }
+  }
+  if (!__any_sync(kAll, span > 0)) return;
+  Quad rv[NV];
+  float st = 0.f;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = rv[v] = Quad{0ull, 0ull};
+  if (span > 0) {
+    st = row_state[key];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) rv[v] = quad_at(tl + (uint64_t)key * row_bytes + col.next(v));
+  }
+  for (int k0 = 0; k0 < span; k0 += KB) {
+    Quad pv[KB][NV];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      // the run's part is in slot 0 of a window whose first position it holds: of all but perhaps the first
+      const float* const src = pl + (int64_t)(k0 + k) * 2 * D + (k0 + k > 0 || first_tail == 0x8000u ? 0 : D);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        pv[k][v] = Quad{0ull, 0ull};
+        if (k0 + k < span) pv[k][v] = quad_at(reinterpret_cast<const char*>(src) + col.next(v));
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < KB; ++k)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = add_quad(acc[v], pv[k][v]);
+  }
+  step(acc, rv, st, key, span > 0);
 }
 
 // ---- (5) rows whose run crosses window edges: add their window partials ---------------------------
@@ -1432,7 +1582,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
 // the group sums are then added in group order.  The association is fixed by the
 // segment's position alone (the order of the list does not matter).
 // FUSE (rows of at most 128 floats): the combined sum is not stored; the row is updated here.
-template <int G, int NV, bool FUSE>
+template <int G, int NV, bool FUSE, bool Wide>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
                     const int32_t* __restrict__ long_list, int nwin, int D, const float* __restrict__ partial,
@@ -1457,7 +1607,7 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
   // block works through its rows one after the other, so that path must stay short -- but a lane group walking a
   // long span is a chain of dependent rounds at the kernel's tail: of 2 / 4 / 8 / 32 / 128 windows, 8 was the
   // fastest (the call 66.7 us against 69.5 with 32 and 89.8 with 128).
-  constexpr int kShort = 8;
+  constexpr int kShort = kShortSpan;
   constexpr int kBatch = NV <= 1 ? 8 : (NV <= 2 ? 4 : 2);
   // The two phases are two chains of dependent loads; with enough blocks the first half of the grid takes the long
   // spans (phase B) and the second half the short ones (phase A), so that the chains run side by side instead of
@@ -1507,7 +1657,7 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
     }
     if (FUSE) {
       const uint32_t key = (uint32_t)uniq[u];
-      if (key < sentinel) adagrad_row_nv<G, NV>(t, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
+      if (key < sentinel) adagrad_row_nv<G, NV, Wide>(t, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
     }
   }
   // phase B: long spans, the whole block per row.  The block owns the list entries blockIdx.x + k*gridDim.x;
@@ -1569,7 +1719,7 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
       }
       if (FUSE) {
         const uint32_t key = (uint32_t)uniq[u];
-        if (key < sentinel) adagrad_row_nv<G, NV>(tt, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
+        if (key < sentinel) adagrad_row_nv<G, NV, Wide>(tt, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
       }
     }
     __syncthreads();
@@ -1648,6 +1798,20 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
   }
 }
 
+// Lanes a window, float4 a lane, halves of the sum-of-squares tree, positions a batch and blocks per SM (of 128 threads: 8 leave
+// a thread 64 registers, 10 leave 48).  A request should cover 128 bytes of a row: groups of 4 lanes with 4 float4 each move rows
+// of 256 bytes at half the rate (random rows of 7 GB: 8.7 G a second, groups of 8 or 16 15.9 G).  More warps beat more requests
+// a warp: 16 float4 in flight a lane, at 120 registers, took 62 us where 8, at 64, take 51.
+template <int G_, int NV_, int H_, int KB_, int kMinBlocks_> struct WindowShape {
+  static constexpr int G = G_, NV = NV_, H = H_, KB = KB_, kMinBlocks = kMinBlocks_;
+};
+// by the float4 a row has, rounded up to a power of two (us of the reduction half, before -> now)
+template <int kQuads> struct WindowShapeFor;
+template <> struct WindowShapeFor<4> { using type = WindowShape<4, 1, 1, 4, 7>; };     // 40 x 32 900 lookups of 16 floats: 104 -> 91
+template <> struct WindowShapeFor<8> { using type = WindowShape<8, 1, 1, 2, 10>; };    // 16 x 43 000 of 32: 42 -> 37
+template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 1, 2, 8>; };    // 26 x 21 500 of 64: 58 -> 51
+template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
+
 template <int G, int NV>
 static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
                           int D, int B, const float* grad, int64_t ld_grad, int col0, float* tables,
@@ -1663,16 +1827,21 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   int32_t* long_list = reinterpret_cast<int32_t*>(ws + p.off_long);
   int32_t* seg = reinterpret_cast<int32_t*>(ws + p.off_seg);
   int32_t* uniq = reinterpret_cast<int32_t*>(ws + p.off_uniq);
-  constexpr bool kFuse = (NV == 1);
-  if (kFuse) {
-    // two float4 per lane (half as many lanes per window) wherever the row has at least eight
-    constexpr int WG = G >= 8 ? G / 2 : G, WNV = G >= 8 ? 2 : 1;
-    constexpr int kWaGroups = kWaThreads / WG;
-    SS_TIMED("window_apply_kernel", st);
-    launch_dependent(window_apply_kernel<WG, WNV>, (unsigned)((p.nwin + kWaGroups - 1) / kWaGroups), kWaThreads, 0, st, 
-        keys, reinterpret_cast<int32_t*>(ws + p.off_sbag), reinterpret_cast<int32_t*>(ws + p.off_uidx), p.L, sentinel,
-        N, D, B, grad, ld_grad, col0, partial, long_list, scalars, p.nwin, (int64_t)umax, d_status, tables, row_state,
-        lr, eps);
+  constexpr bool kFuse = NV == 1, kWide = false;
+  if constexpr (kFuse) {
+    auto window = [&](auto shape) {
+      using S = decltype(shape);
+      constexpr int kPos = kWaThreads / S::G * kWin;
+      SS_TIMED("window_apply_kernel", st);
+      auto go = [&](auto kernel) {
+        launch_dependent(kernel, (unsigned)((p.L + kPos - 1) / kPos), kWaThreads, 0, st, keys, reinterpret_cast<int32_t*>(ws + p.off_sbag),
+                         reinterpret_cast<int32_t*>(ws + p.off_uidx), (int)p.L, sentinel, T, (uint32_t)N, D, B, grad, ld_grad, col0,
+                         partial, long_list, scalars, p.nwin, d_status, tables, row_state, lr, eps);
+      };
+      if (D == S::G * S::NV * 4) go(window_apply_kernel<S::G, S::NV, S::H, S::KB, S::kMinBlocks, true, kWide>);
+      else go(window_apply_kernel<S::G, S::NV, S::H, S::KB, S::kMinBlocks, false, kWide>);
+    };
+    window(typename WindowShapeFor<G * NV>::type());
   } else {
     SS_TIMED("window_reduce_kernel", st);
     launch_dependent(window_reduce_kernel<G, NV>, blocks, 256, 0, st, 
@@ -1683,8 +1852,8 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
     SS_TIMED("combine_rows_kernel", st);
     const int cblocks = p.nwin < num_sms() * 8 ? p.nwin : num_sms() * 8;
     // fused rows of at least eight float4: two float4 per lane, half as many lanes per row, twice as many rows in flight
-    constexpr int CG = (kFuse && G >= 8) ? G / 2 : G, CNV = (kFuse && G >= 8) ? 2 : NV;
-    launch_dependent(combine_rows_kernel<CG, CNV, kFuse>, cblocks, 256, (size_t)(256 / CG) * D * 4, st, 
+    constexpr int CG = (kFuse && !kWide && G >= 8) ? G / 2 : G, CNV = (kFuse && G >= 8) ? 2 : NV;
+    launch_dependent(combine_rows_kernel<CG, CNV, kFuse, kWide>, cblocks, 256, (size_t)(256 / CG) * D * 4, st, 
         seg, scalars, long_list, p.nwin, D, partial, gsum, p.L, sentinel, (int64_t)umax, uniq, tables, row_state, lr, eps);
   }
   if (!kFuse) {

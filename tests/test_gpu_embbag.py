@@ -246,3 +246,57 @@ def test_apply_refuses_a_workspace_sorted_for_another_problem():
     ss.ss_embbag_bwd_apply(dt, ds, T, N, D, B, b1.L, dg, T * D, 0, 0.1, 1e-8, ws, st)
     torch.cuda.synchronize()
     assert int(st.item()) == 0 and not np.array_equal(dt.cpu().numpy(), tables)
+
+
+def _run_lengths_batch(D, lengths, B, seed):
+    """Two tables whose rows are looked up `lengths` times each, cut into B bags at random places (some are empty)."""
+    T, N = 2, len(lengths) + 3
+    cfg = synth.scaled(synth.CONFIGS["tiny"], T=T, N=N, D=D, B=B, bottom=(13, 64, D), top=(3 * D, 64, 1))
+    rng = np.random.default_rng(seed)
+    idx, off = [], [0]
+    for t in range(T):
+        rows = np.repeat(np.arange(len(lengths), dtype=np.int32) + t, lengths)
+        rng.shuffle(rows)
+        cuts = np.sort(rng.integers(0, len(rows) + 1, B - 1))
+        off += list(off[0] + len(idx) + np.append(cuts, len(rows)))
+        idx += list(rows)
+    return cfg, synth.Batch(np.array(idx, np.int32), np.array(off, np.int32), np.zeros((B, 13), np.float32),
+                            np.zeros(B, np.float32))
+
+
+# row widths on both sides of every lane mapping (4, 8, 16, 32 lanes' worth of float4, more than 256 floats), and row
+# frequencies around the window (16 positions), the block's windows, and the longest span that is added beside the window (8)
+@pytest.mark.parametrize("D", [4, 12, 16, 20, 32, 36, 64, 68, 128, 132, 200, 256, 260])
+def test_bwd_runs_around_windows_blocks_and_spans(D):
+    lengths = [15, 1, 16, 16, 32, 17, 128, 1, 127, 2, 144, 7, 113, 1, 129, 3, 1, 1, 1, 260, 12, 33, 111, 1, 5, 600, 31, 96,
+               97, 1, 14, 16, 48, 2, 1, 1, 1040, 30, 18, 112, 113]
+    for seed, extra in ((1, []), (2, [1] * 37), (3, [16] * 33)):
+        cfg, b = _run_lengths_batch(D, extra + lengths, 61, seed)
+        rng = np.random.default_rng(seed)
+        tables = (rng.normal(size=(cfg.T, cfg.N, D)) * 0.05).astype(np.float32)
+        state = (rng.random((cfg.T, cfg.N)) * 1e-4).astype(np.float32)
+        gp = (rng.normal(size=(cfg.B, cfg.T * D)) * 1e-3).astype(np.float32)
+        t_o, s_o = tables.copy(), state.copy()
+        uniq, seg, _ = O.embbag_bwd_adagrad(t_o, s_o, b.indices, b.offsets, cfg.B, gp, cfg.lr, cfg.eps)
+        t_g, s_g, uniq_g, seg_g, _, st = _bwd(cfg, b, tables, state, gp)
+        assert st == 0 and np.array_equal(uniq_g, uniq) and np.array_equal(seg_g, seg)
+        # a row's sum has up to 1040 terms, added in two levels of at most 65 and 16: 81 * 2^-24 = 5e-6 of their size
+        assert_close(t_g - tables, t_o.astype(np.float64) - tables, 3e-5, f"table update, {seed}")
+        assert_close(s_g, s_o, 2e-5, f"row state, {seed}")
+
+
+# bag lengths around the rounds of the gather, odd batches (the last block is not full)
+@pytest.mark.parametrize("D", [4, 16, 20, 32, 64, 68, 128, 132, 200, 256, 260, 512])
+def test_fwd_bags_around_the_rounds_of_the_gather(D):
+    rng = np.random.default_rng(D)
+    T, N, lens = 2, 97, [0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 11, 12, 13, 16, 17, 18, 19, 0, 24, 25, 40, 1, 0]
+    B = len(lens)
+    tables = rng.normal(size=(T, N, D)).astype(np.float32)
+    off = np.concatenate([[0], np.cumsum(lens + lens)]).astype(np.int32)
+    idx = rng.integers(0, N, off[-1]).astype(np.int32)
+    want = O.embbag_fwd(tables, idx, off, B)
+    got, goth, st = _fwd(tables, idx, off, B, col0=0, want_bf16=True)
+    assert st == 0
+    # up to 40 terms of size one added in float: 40 * 2^-24 = 2.4e-6 of the sum's scale, sqrt(40)
+    assert_close(got, want.reshape(B, -1), RTOL_F32, "pooled", floor=1.0)
+    assert np.array_equal(goth, torch.from_numpy(got).to(torch.bfloat16).float().numpy())
