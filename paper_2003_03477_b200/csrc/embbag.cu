@@ -1179,8 +1179,8 @@ __device__ __forceinline__ bool ws_matches(const int32_t* scalars, int64_t L, ui
 // A lane group owns a window of kWin consecutive sorted positions and adds the gradient rows of each
 // run of equal keys in position order.  A run that lies inside the window is complete: its sum goes
 // to gsum[u].  A run that crosses a window edge leaves a partial sum in the window's slot 0 (run
-// covers the window's first position) or slot 1.  This kernel serves rows wider than 128 floats (several
-// float4 per lane); narrower rows take window_apply_kernel, which also updates the rows.
+// covers the window's first position) or slot 1.  This kernel serves rows wider than 256 floats; narrower rows
+// take window_apply_kernel, which also updates the rows.
 template <int G, int NV>
 __global__ void __launch_bounds__(256)
 window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
@@ -1274,7 +1274,7 @@ window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restric
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// ---- (4b) fused window kernel for rows of at most 128 floats --------------------------------------
+// ---- (4b) fused window kernel for rows of at most 256 floats --------------------------------------
 // Same windows and same order of additions as window_reduce_kernel.  A block stages keys and gradient rows of its windows
 // together (32 consecutive positions per warp and round) and requests the table rows of the runs into L2; ballots give the run
 // structure of a window as 16-bit masks.  A batch of positions requests its gradient rows and, for the runs that end in it, the
@@ -1581,7 +1581,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
 // block per row, lane group j adds the partials of windows k0+j, k0+j+groups, ... in ascending order and
 // the group sums are then added in group order.  The association is fixed by the
 // segment's position alone (the order of the list does not matter).
-// FUSE (rows of at most 128 floats): the combined sum is not stored; the row is updated here.
+// FUSE (rows of at most 256 floats): the combined sum is not stored; the row is updated here.
 template <int G, int NV, bool FUSE, bool Wide>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
@@ -1728,10 +1728,8 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
   if (threadIdx.x == 0 && ticket == (int)gridDim.x - 1) { scalars[1] = 0; scalars[kListTicket] = 0; }
 }
 
-// ---- (6) row-wise Adagrad, one lane group per four distinct rows ----------------------------------
+// ---- (6) row-wise Adagrad, one lane group per distinct row (rows of more than 256 floats) ----------------------------------
 //   g = gsum[u];  s = state + mean_d g^2;  row -= lr * g / (sqrt(s) + eps)
-template <int NV> struct RowsPerGroup { static constexpr int value = NV == 1 ? 4 : (NV == 2 ? 2 : 1); };
-
 template <int G, int NV>
 __global__ void __launch_bounds__(256)
 apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ scalars, int D,
@@ -1739,63 +1737,19 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
                   float lr, float eps, int64_t L, uint32_t sentinel, int64_t umax) {
   wait_for_previous_kernel();
   constexpr int kGroups = 256 / G;
-  constexpr int RB = RowsPerGroup<NV>::value;              // rows per group, their loads issued together
   const int grp = threadIdx.x / G, lane = threadIdx.x % G;
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) / G * G));
   if (!ws_matches(scalars, L, sentinel, nullptr)) return;
-  const int U = (int)min((int64_t)scalars[0], umax);
+  const int64_t u = (int64_t)blockIdx.x * kGroups + grp;
+  if (u >= min((int64_t)scalars[0], umax)) return;
+  const uint32_t key = (uint32_t)uniq[u];
+  if (key >= sentinel) return;                             // never true for a consistent workspace
   const int nvec = D >> 2;
-  const int64_t u0 = ((int64_t)blockIdx.x * kGroups + grp) * RB;
-  if (u0 >= U) return;
-  uint32_t key[RB];
-  int64_t urow[RB];
-  bool valid[RB];
+  const float4* p = reinterpret_cast<const float4*>(gsum + u * D);
+  float4 g[NV];
 #pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    valid[r] = u0 + r < U;
-    urow[r] = valid[r] ? u0 + r : 0;
-    if (urow[r] < 0 || urow[r] >= umax) { valid[r] = false; urow[r] = 0; }
-    key[r] = valid[r] ? (uint32_t)uniq[urow[r]] : 0u;
-    if (key[r] >= sentinel) valid[r] = false;              // never true for a consistent workspace
-  }
-  float4 g[RB][NV], rw[RB][NV];
-  float st[RB];
-#pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    const float4* p = reinterpret_cast<const float4*>(gsum + urow[r] * D);
-    const float4* row = reinterpret_cast<const float4*>(tables + (int64_t)key[r] * D);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int c = lane + v * G;
-      g[r][v] = (valid[r] && c < nvec) ? p[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-      rw[r][v] = (valid[r] && c < nvec) ? row[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    st[r] = valid[r] ? row_state[key[r]] : 0.f;
-  }
-#pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    float ss = 0.f;
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-      ss += g[r][v].x * g[r][v].x + g[r][v].y * g[r][v].y + g[r][v].z * g[r][v].z + g[r][v].w * g[r][v].w;
-#pragma unroll
-    for (int off = G / 2; off >= 1; off >>= 1) ss += __shfl_down_sync(gmask, ss, off, G);
-    ss = __shfl_sync(gmask, ss, 0, G);                     // every lane uses lane 0's sum
-    if (!valid[r]) continue;
-    const float s = st[r] + ss / (float)D;
-    const float scale = lr / (sqrtf(s) + eps);
-    float4* row = reinterpret_cast<float4*>(tables + (int64_t)key[r] * D);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int c = lane + v * G;
-      if (c < nvec) {
-        float4 o = rw[r][v];
-        o.x -= scale * g[r][v].x; o.y -= scale * g[r][v].y; o.z -= scale * g[r][v].z; o.w -= scale * g[r][v].w;
-        row[c] = o;
-      }
-    }
-    if (lane == 0) row_state[key[r]] = s;
-  }
+  for (int v = 0; v < NV; ++v) g[v] = lane + v * G < nvec ? p[lane + v * G] : make_float4(0.f, 0.f, 0.f, 0.f);
+  adagrad_row_nv<G, NV, true>(g, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
 }
 
 // Lanes a window, float4 a lane, halves of the sum-of-squares tree, positions a batch and blocks per SM (of 128 threads: 8 leave
@@ -1811,6 +1765,7 @@ template <> struct WindowShapeFor<4> { using type = WindowShape<4, 1, 1, 4, 7>; 
 template <> struct WindowShapeFor<8> { using type = WindowShape<8, 1, 1, 2, 10>; };    // 16 x 43 000 of 32: 42 -> 37
 template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 1, 2, 8>; };    // 26 x 21 500 of 64: 58 -> 51
 template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
+template <> struct WindowShapeFor<64> { using type = WindowShape<32, 2, 1, 2, 6>; };   // 8 x 21 500 of 256: 68 -> 51; 5 x 9 000 of 200: 20 -> 20
 
 template <int G, int NV>
 static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
@@ -1827,7 +1782,7 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   int32_t* long_list = reinterpret_cast<int32_t*>(ws + p.off_long);
   int32_t* seg = reinterpret_cast<int32_t*>(ws + p.off_seg);
   int32_t* uniq = reinterpret_cast<int32_t*>(ws + p.off_uniq);
-  constexpr bool kFuse = NV == 1, kWide = false;
+  constexpr bool kFuse = NV <= 2, kWide = NV == 2;        // (32 lanes hold up to 128 floats with one float4 each)
   if constexpr (kFuse) {
     auto window = [&](auto shape) {
       using S = decltype(shape);
@@ -1856,9 +1811,9 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
     launch_dependent(combine_rows_kernel<CG, CNV, kFuse, kWide>, cblocks, 256, (size_t)(256 / CG) * D * 4, st, 
         seg, scalars, long_list, p.nwin, D, partial, gsum, p.L, sentinel, (int64_t)umax, uniq, tables, row_state, lr, eps);
   }
-  if (!kFuse) {
-    // rows wider than 128 floats: every distinct row is updated from its sum in gsum
-    const uint64_t per_block = (uint64_t)kGroups * RowsPerGroup<NV>::value;
+  if constexpr (!kFuse) {
+    // rows wider than 256 floats: every distinct row is updated from its sum in gsum
+    const uint64_t per_block = (uint64_t)kGroups;
     const unsigned ublocks = (unsigned)((umax + per_block - 1) / per_block);
     SS_TIMED("apply_rows_kernel", st);
     launch_dependent(apply_rows_kernel<G, NV>, ublocks, 256, 0, st, uniq, scalars, D, gsum, tables, row_state, lr, eps, p.L, sentinel,
