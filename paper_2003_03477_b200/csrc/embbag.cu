@@ -1609,10 +1609,14 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
   // fastest (the call 66.7 us against 69.5 with 32 and 89.8 with 128).
   constexpr int kShort = kShortSpan;
   constexpr int kBatch = NV <= 1 ? 8 : (NV <= 2 ? 4 : 2);
-  // The two phases are two chains of dependent loads; with enough blocks the first half of the grid takes the long
-  // spans (phase B) and the second half the short ones (phase A), so that the chains run side by side instead of
-  // one after the other.  A small grid does both in every block.
-  const int nb_long = gridDim.x >= 4 ? (int)gridDim.x / 2 : 0;
+  // The two phases are two chains of dependent loads; with enough blocks the first part of the grid takes the long
+  // spans (phase B) and the rest the short ones (phase A), so that the chains run side by side instead of
+  // one after the other.  A small grid does both in every block.  Half of the grid for each where the window kernel leaves
+  // all crossing runs; behind the fused one few short spans are left, and most of 8 blocks per SM only took other kernels'
+  // places: with 5 per SM, a quarter of them for the short spans, four replicas of the ordinary model take 452 us a round
+  // instead of 455, three of an odd-sized one 104 instead of 106 (the call alone 51 and 51, 93 and 93 for 128 floats; 3 per SM:
+  // 449 and 103, but 54 and 100).
+  const int nb_long = gridDim.x >= 4 ? (FUSE ? (int)gridDim.x * 3 / 4 : (int)gridDim.x / 2) : 0;
   const bool do_short = nb_long == 0 || (int)blockIdx.x >= nb_long;
   const bool do_long = nb_long == 0 || (int)blockIdx.x < nb_long;
   const int a_blk = nb_long == 0 ? (int)blockIdx.x : (int)blockIdx.x - nb_long;
@@ -1805,7 +1809,7 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   }
   {
     SS_TIMED("combine_rows_kernel", st);
-    const int cblocks = p.nwin < num_sms() * 8 ? p.nwin : num_sms() * 8;
+    const int per_sm = kFuse ? 5 : 8, cblocks = p.nwin < num_sms() * per_sm ? p.nwin : num_sms() * per_sm;
     // fused rows of at least eight float4: two float4 per lane, half as many lanes per row, twice as many rows in flight
     constexpr int CG = (kFuse && !kWide && G >= 8) ? G / 2 : G, CNV = (kFuse && G >= 8) ? 2 : NV;
     launch_dependent(combine_rows_kernel<CG, CNV, kFuse, kWide>, cblocks, 256, (size_t)(256 / CG) * D * 4, st, 
