@@ -892,8 +892,7 @@ __device__ __forceinline__ int walk_table(const BucketSort& a, BucketRange& r, u
 
 __device__ __forceinline__ void write_sorted(const SortOut& o, int j, uint32_t key, int pos, int bag, uint32_t u) {
   o.keys[j] = key;
-  o.perm[j] = pos;
-  if (o.perm_out) o.perm_out[j] = pos;
+  if (o.perm_out) o.perm_out[j] = pos;                     // (o.perm is the tiled passes' own)
   o.uidx[j] = (int32_t)u;
   o.sbag[j] = bag;
 }
