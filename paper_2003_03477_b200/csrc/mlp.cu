@@ -12,11 +12,14 @@ namespace ss {
 // Reductions over the batch that are no dense contraction: bias gradients, the gradient of the
 // single-logit layer and of the 13-input layer.  All have the form
 //     out[c * s_cols + j] = sum_b M[b, c] * S[b, j]          (S absent: s_cols = 1, S = 1)
-// One launch takes a list of such jobs.  A block owns 32 columns c and a slice of the batch; its 8
+// One launch takes a list of such jobs.  A block owns 256 or 64 columns c and a slice of the batch; its 8
 // row groups add their rows in ascending order, the groups are added in order, and a second kernel
 // adds the slices in order: every sum has a fixed association.
-// What bounds it is the latency of a block's loads, so a thread keeps 8 rows (of 8 columns) or 16 rows (of one) in flight:
-// with 4 it took 13.8 / 34 us (the sums of the 2048- and the 4096-sample model), now 8.5 / 28.
+// What bounds it is the latency of a block's loads, so a thread keeps 8 rows (of 8 columns) or 16 rows (of two) in flight:
+// with 4 it took 13.8 / 34 us (the sums of the 2048- and the 4096-sample model), with 8 and 16 rows 8.5 / 28.  The first layer's
+// gradient takes two columns a thread (a row of S read from shared memory serves both; its loads start while the S tile is
+// filled) and all threads add the row groups: half as many blocks, of which three fit beside a tensor-core CTA.  28 -> 24 us for
+// the 4096-sample model, the same for the other, but four replicas of it take 455 us a round instead of 460.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxJobs = 2 * kMaxLayers + 2;
 constexpr int kMaxSCols = 16;
@@ -43,6 +46,7 @@ __device__ __forceinline__ float load_kind(const void* p, int kind, int64_t i) {
 
 constexpr int kRedRows = 256;     // most rows of the batch a block takes (bounds the staged S tile)
 constexpr int kRedWide = 256;     // columns per block of a job without a second factor matrix (s_cols = 1)
+constexpr int kRedPairs = 64;     // columns per block of a job with one
 
 // Eight consecutive elements M[row, c .. c+7] as floats; elements at or beyond ncols read as zero.  One
 // 128-bit load (bf16) or two (float) when the address allows it, element loads otherwise.
@@ -72,22 +76,51 @@ __device__ __forceinline__ void load8_kind(const void* p, int kind, int64_t row,
   }
 }
 
-__global__ void __launch_bounds__(256)
+// Rows ry, ry + 8, ... of two neighbouring columns, in ascending order, times the rows of S in s_tile: F rows in flight, the
+// first ones while stage() fills s_tile.
+template <int F, typename Raw, typename Stage, typename Load, typename Value>
+__device__ __forceinline__ void two_column_sums(const float* s_tile, int ry, int nrows, float (&acc)[2][kMaxSCols], Stage stage, Load load,
+                                                Value value) {
+  Raw m[F];
+  auto fetch = [&](int rr) {
+#pragma unroll
+    for (int u = 0; u < F; ++u) m[u] = rr + 8 * u < nrows ? load(rr + 8 * u) : Raw{};
+  };
+  fetch(ry);
+  stage();
+  for (int rr = ry; rr < nrows; rr += 8 * F) {
+    if (rr != ry) fetch(rr);
+#pragma unroll
+    for (int u = 0; u < F; ++u) {
+      if (rr + 8 * u >= nrows) break;
+      const float2 v = value(m[u]);
+      const float4* srow = reinterpret_cast<const float4*>(s_tile + (rr + 8 * u) * kMaxSCols);
+#pragma unroll
+      for (int q4 = 0; q4 < kMaxSCols / 4; ++q4) {
+        const float4 sv = srow[q4];                            // one 128-bit broadcast read for four columns of S
+        const float sq[4] = {sv.x, sv.y, sv.z, sv.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          acc[0][4 * q4 + k] = fmaf(v.x, sq[k], acc[0][4 * q4 + k]);
+          acc[1][4 * q4 + k] = fmaf(v.y, sq[k], acc[1][4 * q4 + k]);
+        }
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256, 3)
 batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int rows_per_split, float* __restrict__ partial) {
   wait_for_previous_kernel();
   // S rows of this block's batch slice, as float; then the row groups' sums (8 x 256 or 8 x 32 x 17 floats)
   constexpr int kPartFloats = 8 * 32 * (kMaxSCols + 1);
   static_assert(kPartFloats >= kRedRows * kMaxSCols && kPartFloats >= 8 * kRedWide, "one buffer serves all three uses");
   __shared__ __align__(16) float s_tile[kPartFloats];
-  __shared__ RedJob s_job;
-  if (threadIdx.x == 0) {
-    int j = 0;
-    while (j + 1 < jobs.njobs && (int)blockIdx.x >= jobs.job[j + 1].tile0) ++j;
-    s_job = jobs.job[j];
-  }
-  __syncthreads();
-  const RedJob J = s_job;                                    // the job's fields in registers
   const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
+  // the last job that begins at or before this column tile: every warp finds it by itself
+  int begun = 0;
+  for (int j = cx; j < jobs.njobs; j += 32) begun += (int)blockIdx.x >= jobs.job[j].tile0;
+  const RedJob J = jobs.job[__reduce_add_sync(0xffffffffu, begun) - 1];
   const int sc = J.s_cols;
   const int r0 = blockIdx.y * rows_per_split;
   const int r1 = min(B, r0 + rows_per_split);
@@ -170,53 +203,53 @@ batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int row
     return;
   }
 
-  // ---- a second factor with several columns (the layer with few inputs): 32 columns c per block, each thread
-  // keeps one sum per column of S
-  const int c = ((int)blockIdx.x - J.tile0) * 32 + cx;
-  // S rows as float, padded with zeros to kMaxSCols columns so that the inner product needs no column test
-  for (int i = threadIdx.x; i < nrows * kMaxSCols; i += 256) {
-    const int rr = i / kMaxSCols, q = i % kMaxSCols;
-    s_tile[i] = q < sc ? load_kind(J.S, J.s_kind, (int64_t)(r0 + rr) * J.lds + q) : 0.f;
-  }
-  __syncthreads();
-  float acc[kMaxSCols];
+  // ---- a second factor with several columns (the layer with few inputs): 64 columns c per block, two neighbours a thread,
+  // which keeps one sum per column of S for each; a row of S read from shared memory serves both
+  const int c = ((int)blockIdx.x - J.tile0) * kRedPairs + 2 * cx;
+  float acc[2][kMaxSCols];
 #pragma unroll
-  for (int q = 0; q < kMaxSCols; ++q) acc[q] = 0.f;
-  if (c < J.ncols) {
-    // sixteen rows of M in flight per thread; rows are added in ascending order
-    for (int rr = ry; rr < nrows; rr += 128) {
-      float m[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u)
-        m[u] = (rr + 8 * u < nrows) ? load_kind(J.M, J.m_kind, (int64_t)(r0 + rr + 8 * u) * J.ldm + c) : 0.f;
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        if (rr + 8 * u < nrows) {
-          const float4* srow = reinterpret_cast<const float4*>(s_tile + (rr + 8 * u) * kMaxSCols);
-#pragma unroll
-          for (int q4 = 0; q4 < kMaxSCols / 4; ++q4) {
-            const float4 sv = srow[q4];                    // one 128-bit broadcast read for four columns
-            acc[4 * q4 + 0] = fmaf(m[u], sv.x, acc[4 * q4 + 0]);
-            acc[4 * q4 + 1] = fmaf(m[u], sv.y, acc[4 * q4 + 1]);
-            acc[4 * q4 + 2] = fmaf(m[u], sv.z, acc[4 * q4 + 2]);
-            acc[4 * q4 + 3] = fmaf(m[u], sv.w, acc[4 * q4 + 3]);
-          }
-        }
-      }
+  for (int q = 0; q < kMaxSCols; ++q) acc[0][q] = acc[1][q] = 0.f;
+  auto stage = [&] {
+    // S rows as float, padded with zeros to kMaxSCols columns so that the inner product needs no column test
+    for (int i = threadIdx.x; i < nrows * kMaxSCols; i += 256) {
+      const int rr = i / kMaxSCols, q = i % kMaxSCols;
+      s_tile[i] = q < sc ? load_kind(J.S, J.s_kind, (int64_t)(r0 + rr) * J.lds + q) : 0.f;
     }
+    __syncthreads();
+  };
+  if (J.m_kind == OP_BF16 && (J.ldm & 1) == 0 && (J.ncols & 1) == 0 && (reinterpret_cast<uintptr_t>(J.M) & 3u) == 0) {
+    const __nv_bfloat16* M = reinterpret_cast<const __nv_bfloat16*>(J.M) + (int64_t)r0 * J.ldm + c;
+    two_column_sums<16, uint32_t>(
+        s_tile, ry, nrows, acc, stage,
+        [&](int r) { return c < J.ncols ? *reinterpret_cast<const uint32_t*>(M + (int64_t)r * J.ldm) : 0u; },
+        [](uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); });   // a bf16 is the upper half of a float
+  } else {
+    two_column_sums<8, float2>(
+        s_tile, ry, nrows, acc, stage,
+        [&](int r) {
+          const int64_t i = (int64_t)(r0 + r) * J.ldm + c;
+          return make_float2(c < J.ncols ? load_kind(J.M, J.m_kind, i) : 0.f, c + 1 < J.ncols ? load_kind(J.M, J.m_kind, i + 1) : 0.f);
+        },
+        [](float2 v) { return v; });
   }
-  __syncthreads();                                           // the S tile is no longer read
+  __syncthreads();                                             // the S tile is no longer read
+  // the even columns of the block, then the odd ones: half the buffer, and a block fits beside a tensor-core CTA
   float (*part)[32][kMaxSCols + 1] = reinterpret_cast<float (*)[32][kMaxSCols + 1]>(s_tile);   // [8][32][17]
+  const int c0 = ((int)blockIdx.x - J.tile0) * kRedPairs;
+  float* dst = partial + (int64_t)blockIdx.y * jobs.total + J.part_off;
 #pragma unroll
-  for (int q = 0; q < kMaxSCols; ++q) part[ry][cx][q] = acc[q];
-  __syncthreads();
-  if (ry == 0 && c < J.ncols) {
-    float* dst = partial + (int64_t)blockIdx.y * jobs.total + J.part_off + (int64_t)c * sc;
-    for (int q = 0; q < sc; ++q) {
+  for (int h = 0; h < 2; ++h) {
+    if (h > 0) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kMaxSCols; ++q) part[ry][cx][q] = acc[h][q];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 32 * sc; i += 256) {
+      const int col = i / sc, q = i - col * sc, co = c0 + 2 * col + h;
+      if (co >= J.ncols) break;
       float t = 0.f;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) t += part[r][cx][q];
-      dst[q] = t;
+      for (int r = 0; r < 8; ++r) t += part[r][col][q];
+      dst[(int64_t)co * sc + q] = t;
     }
   }
 }
@@ -789,7 +822,7 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
     J.M = M; J.m_kind = m_kind; J.ldm = ldm; J.ncols = ncols;
     J.S = S; J.s_kind = s_kind; J.lds = lds; J.s_cols = s_cols;
     J.tile0 = jobs.ntiles; J.part_off = jobs.total; J.out_off = out_off;
-    jobs.ntiles += s_cols == 1 ? (ncols + kRedWide - 1) / kRedWide : (ncols + 31) / 32;
+    jobs.ntiles += s_cols == 1 ? (ncols + kRedWide - 1) / kRedWide : (ncols + kRedPairs - 1) / kRedPairs;
     jobs.total += ncols * s_cols;
   };
 
