@@ -8,8 +8,8 @@
 // Backward: (1-3) stable LSD radix sort by key t*N+row, unique keys and segment offsets, in one launch: ranges of each
 // table in shared memory, or, for tables too long or too skewed for that, tiled passes over all SMs; (4) the sorted lookups are cut into windows of 16 consecutive positions; a lane group
 // sums the gradients of each run of equal keys inside its window in position order.  A run that
-// lies inside one window is final and is updated at once; a run that crosses a window edge leaves a
-// partial sum, and a second kernel adds the partials of such a row in window order and updates it.
+// lies inside one window is final and is updated at once; a run that crosses a window edge leaves
+// partial sums, added in window order by the group in which it starts, or by a second kernel where the run leaves the block.
 // Work per group is the same whatever the skew of the row distribution, and every sum has a fixed
 // association, so results do not depend on scheduling.
 #include "common.cuh"
@@ -98,6 +98,71 @@ embbag_fwd_kernel(const float* __restrict__ tables, int T, uint32_t N, int D,
   if (bad && d_status) atomicOr(d_status, bad);
 }
 
+// Rows of 65 to 256 floats, many bags: a block takes a stretch of consecutive bags, and the blocks that land on an SM at launch
+// take neighbouring stretches, so an SM stays with one table and finds its popular rows in L1; with half of the threads there
+// are enough registers for every row of a round to be in flight.  What bounds the form above there is the latency of rows from
+// L2, half of which another SM has just read as well.  us alone (L2 flushed), before -> now: 26 tables x 65 600 lookups of 128
+// floats 84 -> 74, 26 x 32 800 52 -> 45, 8 x 21 500 of 256 floats 33 -> 29.  1536 threads an SM at 40 registers: 121 and 68;
+// narrower rows gain nothing (64 floats 28.7 -> 30, 16 floats 45 -> 47), and beside other replicas' kernels they lose.
+constexpr int kStretchThreads = 512, kStretchBlocks = 2;   // blocks per SM
+template <int G>
+__global__ void __launch_bounds__(kStretchThreads, kStretchBlocks)
+embbag_fwd_stretch_kernel(const float* __restrict__ tables, int T, uint32_t N, int D,
+                          const int32_t* __restrict__ indices, const int32_t* __restrict__ offsets, int B,
+                          float* __restrict__ out_f32, int64_t ld_f32,
+                          __nv_bfloat16* __restrict__ out_bf16, int64_t ld_bf16, int col0,
+                          int sms, int per_block, int32_t* __restrict__ d_status) {
+  wait_for_previous_kernel();
+  constexpr int kGroups = kStretchThreads / G, NV = 2, kRows = 4;
+  const int grp = threadIdx.x / G, lane = threadIdx.x % G;
+  const int64_t bags = (int64_t)T * B;
+  const int64_t first = (int64_t)((int)blockIdx.x % sms * kStretchBlocks + (int)blockIdx.x / sms) * per_block;
+  const int64_t end = min(bags, first + per_block);
+  if (first >= end) return;
+  const int L = __ldg(offsets + bags);
+  const uint32_t nvec = (uint32_t)D >> 2;
+  int t = (int)(first / B), b = (int)(first - (int64_t)t * B) + grp, bad = 0;
+  for (int64_t i = first + grp; i < end; i += kGroups, b += kGroups) {
+    while (b >= B) { b -= B; ++t; }
+    int lo = offsets[i], hi = offsets[i + 1];
+    if (lo < 0 || hi < lo || hi > L) { bad |= SS_DEV_BAD_OFFSET; lo = hi = 0; }   // as above: an empty bag
+    const float4* tab = reinterpret_cast<const float4*>(tables + (int64_t)t * N * D);
+    float4 acc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = lo; j < hi; j += kRows) {
+      uint32_t idx[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) idx[u] = (j + u < hi) ? (uint32_t)__ldg(indices + j + u) : 0xffffffffu;
+      float4 rowv[kRows][NV];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const bool ok = idx[u] < N;
+        if (!ok && j + u < hi) bad |= SS_DEV_BAD_INDEX;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const uint32_t c = lane + v * G;
+          rowv[u][v] = (ok && c < nvec) ? __ldg(tab + (idx[u] * nvec + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = add4(acc[v], rowv[u][v]);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int c = lane + v * G;
+      if (c < (int)nvec) {
+        const int64_t col = (int64_t)col0 + (int64_t)t * D + 4 * c;
+        if (out_f32) *reinterpret_cast<float4*>(out_f32 + (int64_t)b * ld_f32 + col) = acc[v];
+        if (out_bf16) *reinterpret_cast<uint2*>(out_bf16 + (int64_t)b * ld_bf16 + col) = bf16x4(acc[v]);
+      }
+    }
+  }
+  if (bad && d_status) atomicOr(d_status, bad);
+}
+
 template <int G, int NV>
 static void launch_fwd(const float* tables, int T, int64_t N, int D, const int32_t* indices,
                        const int32_t* offsets, int B, float* out_f32, int64_t ld_f32, __nv_bfloat16* out_bf16,
@@ -105,6 +170,16 @@ static void launch_fwd(const float* tables, int T, int64_t N, int D, const int32
   // rows of 65..128 floats: two float4 per lane and 16 lanes per bag (measured faster than 32 lanes with one each;
   // for narrower rows the single-float4 form is the faster one)
   constexpr int FG = (NV == 1 && G == 32) ? 16 : G, FNV = (NV == 1 && G == 32) ? 2 : NV;
+  if constexpr (FNV == 2) {
+    // from the point on where the bags fill every SM once, two of them or more for a lane group of a stretch
+    const int64_t bags = (int64_t)T * B, grid = (int64_t)num_sms() * kStretchBlocks;
+    if (bags * FG >= 2048ll * num_sms()) {
+      SS_TIMED("embbag_fwd_kernel", st);
+      launch_dependent(embbag_fwd_stretch_kernel<FG>, (unsigned)grid, kStretchThreads, 0, st, tables, T, (uint32_t)N, D, indices, offsets,
+                       B, out_f32, ld_f32, out_bf16, ld_bf16, col0, num_sms(), (int)((bags + grid - 1) / grid), d_status);
+      return;
+    }
+  }
   const int per_block = 256 / FG;
   const dim3 blocks((unsigned)((B + per_block - 1) / per_block), (unsigned)T);
   { SS_TIMED("embbag_fwd_kernel", st);

@@ -300,3 +300,42 @@ def test_fwd_bags_around_the_rounds_of_the_gather(D):
     # up to 40 terms of size one added in float: 40 * 2^-24 = 2.4e-6 of the sum's scale, sqrt(40)
     assert_close(got, want.reshape(B, -1), RTOL_F32, "pooled", floor=1.0)
     assert np.array_equal(goth, torch.from_numpy(got).to(torch.bfloat16).float().numpy())
+
+
+# a call with enough bags for the form whose blocks take stretches of consecutive bags (rows of 65 to 256 floats): stretches
+# that end inside a table, an odd batch, empty bags, and batches smaller than a block's lane groups (many tables)
+@pytest.mark.parametrize("D,T", [(64, 7), (68, 600), (100, 2), (128, 7), (132, 5), (200, 1200), (256, 3)])
+def test_fwd_stretches_of_bags_match_the_sum_of_their_rows(D, T):
+    lanes = 16 if D <= 128 else 32
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = sms * 2048 // lanes // T + 3
+    g = torch.Generator(device="cuda").manual_seed(D)
+    N = 61
+    tables = torch.randn(T, N, D, generator=g, device="cuda")
+    lens = torch.randint(0, 9, (T * B,), generator=g, device="cuda")
+    off = torch.zeros(T * B + 1, dtype=torch.int64, device="cuda")
+    torch.cumsum(lens, 0, out=off[1:])
+    idx = torch.randint(0, N, (int(off[-1]),), generator=g, device="cuda")
+    table = torch.repeat_interleave(torch.arange(T * B, device="cuda") // B, lens)
+    want = torch.nn.functional.embedding_bag(idx + table * N, tables.double().view(T * N, D), off, mode="sum", include_last_offset=True)
+    out = torch.full((B, T * D + 4), -7.0, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    i32, o32 = idx.int(), off.int()
+    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D + 4, None, 0, 4, st)
+    assert int(st.item()) == 0 and bool((out[:, :4] == -7.0).all())
+    got = out[:, 4:].view(B, T, D).transpose(0, 1).reshape(T * B, D).double()
+    # up to 8 terms of size one: 8 * 2^-24 of the sum of their magnitudes, at most 8 * 5
+    assert float((got - want).abs().max()) <= 2e-5
+    # an index outside a table and a decreasing offset: skipped, and said so; the other bags are as before
+    bags = torch.nonzero(lens > 1).flatten()
+    bad_bag, cut = int(bags[0]), int(bags[len(bags) // 2])
+    i32[int(off[bad_bag])] = N
+    o32[cut + 1] = o32[cut] - 1
+    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D + 4, None, 0, 4, st)
+    assert int(st.item()) == ss.SS_DEV_BAD_INDEX | ss.SS_DEV_BAD_OFFSET
+    again = out[:, 4:].view(B, T, D).transpose(0, 1).reshape(T * B, D).double()
+    rest = want[bad_bag] - tables[bad_bag // B, idx[off[bad_bag]]].double()
+    assert float((again[bad_bag] - rest).abs().max()) <= 2e-5 and not bool(again[cut].any())
+    same = torch.ones(T * B, dtype=torch.bool, device="cuda")
+    same[[bad_bag, cut, cut + 1]] = False
+    assert torch.equal(again[same], got[same])
