@@ -320,9 +320,11 @@ def test_fwd_stretches_of_bags_match_the_sum_of_their_rows(D, T):
     want = torch.nn.functional.embedding_bag(idx + table * N, tables.double().view(T * N, D), off, mode="sum", include_last_offset=True)
     out = torch.full((B, T * D + 4), -7.0, device="cuda")
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    outh = torch.full((B, T * D + 12), -7.0, dtype=torch.bfloat16, device="cuda")
     i32, o32 = idx.int(), off.int()
-    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D + 4, None, 0, 4, st)
-    assert int(st.item()) == 0 and bool((out[:, :4] == -7.0).all())
+    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D + 4, outh, T * D + 12, 4, st)
+    assert int(st.item()) == 0 and bool((out[:, :4] == -7.0).all()) and bool((outh[:, :4] == -7.0).all())
+    assert torch.equal(outh[:, 4:4 + T * D], out[:, 4:].bfloat16()) and bool((outh[:, 4 + T * D:] == -7.0).all())
     got = out[:, 4:].view(B, T, D).transpose(0, 1).reshape(T * B, D).double()
     # up to 8 terms of size one: 8 * 2^-24 of the sum of their magnitudes, at most 8 * 5
     assert float((got - want).abs().max()) <= 2e-5
