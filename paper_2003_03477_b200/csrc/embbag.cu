@@ -1917,13 +1917,16 @@ __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_f
 // Whether the bucket sort takes a problem, how many lookups it gives a range, and the most ranges there can be, whatever the
 // tables' lengths: a block for each.  Every further range reads the index list once more and holds an SM, so a table gets as
 // few ranges as hold its lookups (four replicas of the ordinary model 478 us a round with two ranges a table, 494 with three).
-// Few tables are cut finer, down to 5500 lookups a range, while that takes no more than a quarter of the SMs (5 tables of
-// 9000 lookups: 91 -> 79 us for lookup and update).  Blocks without a range cost nothing that could be measured.
-static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, BucketSort* a, int64_t* blocks, int* nb) {
+// Few tables are cut finer: down to 5500 lookups a range, while that takes no more than a quarter of the SMs, where the sort is
+// a call by itself, which runs beside other work (three replicas of 11 tables of 10 700 lookups 104 us a round; 107 with 2750 a
+// range, 121 with 1400 and half of the SMs); down to 1400, on half of them, where the update waits for the sort in the same call
+// (5 tables of 9000 lookups 26 -> 21.5 us, lookup and update 60 -> 55; 12 of 10 700 27 -> 22).  Blocks without a range cost
+// nothing that could be measured.
+static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, bool waited_for, BucketSort* a, int64_t* blocks, int* nb) {
   const int64_t avg = (L + T - 1) / T;
   if (B > 65535 || avg > 44000) return false;              // bag numbers, plus one, take 16 bits
   int64_t C = (avg + kBsRange - 1) / kBsRange;
-  const int64_t fine = (avg + 5499) / 5500, room = num_sms() / 4 / T;
+  const int64_t least = waited_for ? 1400 : 5500, fine = (avg + least - 1) / least, room = num_sms() / (waited_for ? 2 : 4) / T;
   a->per_range = kBsRange;
   if (C < fine && C < room) {
     C = fine < room ? fine : room;
@@ -2060,7 +2063,7 @@ static ss_status bwd_impl(bool do_sort, bool do_apply, float* tables, float* row
     BucketSort bs{};
     int64_t blocks = 0;
     int nb = 0;
-    const bool bucket = plan_bucket_sort(T, N, B, L, &bs, &blocks, &nb);
+    const bool bucket = plan_bucket_sort(T, N, B, L, do_apply, &bs, &blocks, &nb);
     stt = clear_words(ctl, kCtlCounts + (bucket ? T * kBsMaxBuckets : 0), cs);
     if (stt != SS_OK) return stt;
     if (bucket) {

@@ -111,3 +111,35 @@ def test_sort_skips_malformed_lookups_in_every_form(B, bag):
     uniq, seg, got, st = _sort(T, N, B, idx, off2)
     assert st == ss.SS_DEV_BAD_OFFSET
     assert np.array_equal(np.sort(got), np.arange(idx.size))
+
+
+# the form whose update waits for the sort cuts few tables finer: 1400 lookups a range, up to eight ranges, half of the SMs
+@pytest.mark.parametrize("T,N,B,bag,rows", [
+    (1, 50_000, 1400, 1, UNIFORM), (1, 50_000, 1401, 1, UNIFORM),       # one range, two
+    (3, 1000, 700, 16, UNIFORM), (5, 300_007, 1500, 6, HOT_LOW), (1, 5, 2000, 10, UNIFORM),   # eight ranges; fewer rows than ranges
+    (2, 100_000, 4000, 8, ONE_ROW(0.8, 0.6)), (12, 20_000, 1000, 10, HOT_LOW), (74, 900, 200, 8, UNIFORM),
+])
+def test_sort_that_the_update_waits_for(T, N, B, bag, rows):
+    rng = np.random.default_rng(T * 1000 + N + B)
+    lens = np.full(T * B, bag)
+    off, D = _offsets(lens), 4
+    idx = rows(N)(rng, int(off[-1]))
+    keys = (np.repeat(np.arange(T * B) // B, lens)).astype(np.int64) * N + idx
+    perm = np.argsort(keys, kind="stable")
+    uniq = np.unique(keys)
+    L = idx.size
+    i32 = dict(dtype=torch.int32, device="cuda")
+    ws = torch.randint(0, 255, (ss.ss_embbag_bwd_workspace_bytes(T, N, D, B, L),), dtype=torch.uint8, device="cuda")
+    u, s, p = (torch.full((L + 1,), -1, **i32) for _ in range(3))
+    num, st = torch.full((1,), -1, **i32), torch.zeros(1, **i32)
+    tables, state, grad = torch.zeros(T, N, D, device="cuda"), torch.ones(T * N, device="cuda"), torch.ones(B, T * D, device="cuda")
+    ss.ss_embbag_bwd_adagrad(tables, state, T, N, D, torch.from_numpy(idx.astype(np.int32)).cuda(), torch.from_numpy(off.astype(np.int32)).cuda(),
+                             B, L, grad, T * D, 0, 0.0, 1e-8, ws, u, s, p, num, st)
+    assert int(st.item()) == 0 and int(num.item()) == len(uniq)
+    assert int(ws[-(-(32 + 32 * T) // 256) * -256:][:4].view(torch.int32).item()) == 0        # no tiled passes
+    assert np.array_equal(p.cpu().numpy()[:L], perm) and np.array_equal(u.cpu().numpy()[:len(uniq)], uniq)
+    counts = np.bincount(keys.astype(np.int64), minlength=T * N).astype(np.float64)
+    assert np.array_equal(np.diff(s.cpu().numpy()[:len(uniq) + 1]), counts[uniq])
+    # every lookup brings a gradient of ones: the state grows by the square of the count, exact in float up to 2^24
+    got = state.cpu().numpy().astype(np.float64)
+    assert np.allclose(got, 1.0 + counts ** 2, rtol=2.0 ** -23, atol=0)
