@@ -12,6 +12,7 @@
 // partial sums, added in window order by the group in which it starts, or by a second kernel where the run leaves the block.
 // Work per group is the same whatever the skew of the row distribution, and every sum has a fixed
 // association, so results do not depend on scheduling.
+#include <type_traits>
 #include "common.cuh"
 #include "profile.cuh"
 
@@ -1253,8 +1254,8 @@ __device__ __forceinline__ bool ws_matches(const int32_t* scalars, int64_t L, ui
 // A lane group owns a window of kWin consecutive sorted positions and adds the gradient rows of each
 // run of equal keys in position order.  A run that lies inside the window is complete: its sum goes
 // to gsum[u].  A run that crosses a window edge leaves a partial sum in the window's slot 0 (run
-// covers the window's first position) or slot 1.  This kernel serves rows wider than 256 floats; narrower rows
-// take window_apply_kernel, which also updates the rows.
+// covers the window's first position) or slot 1.  This kernel serves rows wider than 256 floats, and of
+// more than 128 where the windows are few; the others take window_apply_kernel, which also updates the rows.
 template <int G, int NV>
 __global__ void __launch_bounds__(256)
 window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
@@ -1806,7 +1807,7 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
   if (threadIdx.x == 0 && ticket == (int)gridDim.x - 1) { scalars[1] = 0; scalars[kListTicket] = 0; }
 }
 
-// ---- (6) row-wise Adagrad, one lane group per distinct row (rows of more than 256 floats) ----------------------------------
+// ---- (6) row-wise Adagrad, one lane group per distinct row (what window_reduce_kernel summed) ----------------------------------
 //   g = gsum[u];  s = state + mean_d g^2;  row -= lr * g / (sqrt(s) + eps)
 template <int G, int NV>
 __global__ void __launch_bounds__(256)
@@ -1845,8 +1846,8 @@ template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 1, 2, 8>;
 template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
 template <> struct WindowShapeFor<64> { using type = WindowShape<32, 2, 1, 2, 6>; };   // 8 x 21 500 of 256: 68 -> 51; 5 x 9 000 of 200: 20 -> 20
 
-template <int G, int NV>
-static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
+template <int G, int NV, bool kFuse>
+static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
                           int D, int B, const float* grad, int64_t ld_grad, int col0, float* tables,
                           float* row_state, float lr, float eps, int32_t* d_status, cudaStream_t st) {
   constexpr int kGroups = 256 / G;
@@ -1860,7 +1861,7 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   int32_t* long_list = reinterpret_cast<int32_t*>(ws + p.off_long);
   int32_t* seg = reinterpret_cast<int32_t*>(ws + p.off_seg);
   int32_t* uniq = reinterpret_cast<int32_t*>(ws + p.off_uniq);
-  constexpr bool kFuse = NV <= 2, kWide = NV == 2;        // (32 lanes hold up to 128 floats with one float4 each)
+  constexpr bool kWide = NV == 2;                          // (32 lanes hold up to 128 floats with one float4 each)
   if constexpr (kFuse) {
     auto window = [&](auto shape) {
       using S = decltype(shape);
@@ -1890,13 +1891,32 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
         seg, scalars, long_list, p.nwin, D, partial, gsum, p.L, sentinel, (int64_t)umax, uniq, tables, row_state, lr, eps);
   }
   if constexpr (!kFuse) {
-    // rows wider than 256 floats: every distinct row is updated from its sum in gsum
+    // every distinct row is updated from its sum in gsum
     const uint64_t per_block = (uint64_t)kGroups;
     const unsigned ublocks = (unsigned)((umax + per_block - 1) / per_block);
     SS_TIMED("apply_rows_kernel", st);
     launch_dependent(apply_rows_kernel<G, NV>, ublocks, 256, 0, st, uniq, scalars, D, gsum, tables, row_state, lr, eps, p.L, sentinel,
                                                       (int64_t)umax);
   }
+}
+
+// Rows of up to 128 floats are updated from the window kernel, wider ones than 256 from their sums in memory; in between it
+// depends on how many windows there are: a lane group of the fused kernel works through its 16 positions in eight dependent
+// rounds, which takes the time where the windows are few (lookup and update of 26 tables x 90 lookups of 248 floats: fused 34 us,
+// not fused 31), while the sums' way through memory does where they fill the SMs (8 x 21 500 of 256 floats 51 and 68 us, the
+// update alone; 5 x 9000 of 200, 19 windows an SM, 20 and 20).
+constexpr int kFuseWindows = 16;                           // per SM
+template <int G, int NV>
+static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
+                          int D, int B, const float* grad, int64_t ld_grad, int col0, float* tables,
+                          float* row_state, float lr, float eps, int32_t* d_status, cudaStream_t st) {
+  auto as = [&](auto fuse) {
+    launch_reduce_as<G, NV, decltype(fuse)::value>(p, ws, keys, T, N, D, B, grad, ld_grad, col0, tables, row_state, lr, eps, d_status, st);
+  };
+  if constexpr (NV == 1) as(std::true_type());
+  else if constexpr (NV > 2) as(std::false_type());
+  else if (p.nwin >= kFuseWindows * num_sms()) as(std::true_type());
+  else as(std::false_type());
 }
 
 #define SS_DISPATCH_GNV(D_, CALL)                                                 \
