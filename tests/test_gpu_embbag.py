@@ -268,21 +268,35 @@ def _run_lengths_batch(D, lengths, B, seed):
 # frequencies around the window (16 positions), the block's windows, and the longest span that is added beside the window (8)
 @pytest.mark.parametrize("D", [4, 12, 16, 20, 32, 36, 64, 68, 128, 132, 200, 256, 260])
 def test_bwd_runs_around_windows_blocks_and_spans(D):
-    lengths = [15, 1, 16, 16, 32, 17, 128, 1, 127, 2, 144, 7, 113, 1, 129, 3, 1, 1, 1, 260, 12, 33, 111, 1, 5, 600, 31, 96,
-               97, 1, 14, 16, 48, 2, 1, 1, 1040, 30, 18, 112, 113]
     for seed, extra in ((1, []), (2, [1] * 37), (3, [16] * 33)):
-        cfg, b = _run_lengths_batch(D, extra + lengths, 61, seed)
-        rng = np.random.default_rng(seed)
-        tables = (rng.normal(size=(cfg.T, cfg.N, D)) * 0.05).astype(np.float32)
-        state = (rng.random((cfg.T, cfg.N)) * 1e-4).astype(np.float32)
-        gp = (rng.normal(size=(cfg.B, cfg.T * D)) * 1e-3).astype(np.float32)
-        t_o, s_o = tables.copy(), state.copy()
-        uniq, seg, _ = O.embbag_bwd_adagrad(t_o, s_o, b.indices, b.offsets, cfg.B, gp, cfg.lr, cfg.eps)
-        t_g, s_g, uniq_g, seg_g, _, st = _bwd(cfg, b, tables, state, gp)
-        assert st == 0 and np.array_equal(uniq_g, uniq) and np.array_equal(seg_g, seg)
-        # a row's sum has up to 1040 terms, added in two levels of at most 65 and 16: 81 * 2^-24 = 5e-6 of their size
-        assert_close(t_g - tables, t_o.astype(np.float64) - tables, 3e-5, f"table update, {seed}")
-        assert_close(s_g, s_o, 2e-5, f"row state, {seed}")
+        _check_runs(D, extra + RUN_LENGTHS, seed)
+
+
+# rows of 129 to 256 floats once more with as many windows as the fused kernel wants (16 an SM)
+@pytest.mark.parametrize("D", [132, 200, 256])
+def test_bwd_runs_of_wide_rows_with_many_windows(D):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    repeats = -(-16 * sms * 16 // (2 * sum(RUN_LENGTHS))) + 1
+    _check_runs(D, [5] + RUN_LENGTHS * repeats, 4)
+
+
+RUN_LENGTHS = [15, 1, 16, 16, 32, 17, 128, 1, 127, 2, 144, 7, 113, 1, 129, 3, 1, 1, 1, 260, 12, 33, 111, 1, 5, 600, 31, 96,
+               97, 1, 14, 16, 48, 2, 1, 1, 1040, 30, 18, 112, 113]
+
+
+def _check_runs(D, lengths, seed):
+    cfg, b = _run_lengths_batch(D, lengths, 61, seed)
+    rng = np.random.default_rng(seed)
+    tables = (rng.normal(size=(cfg.T, cfg.N, D)) * 0.05).astype(np.float32)
+    state = (rng.random((cfg.T, cfg.N)) * 1e-4).astype(np.float32)
+    gp = (rng.normal(size=(cfg.B, cfg.T * D)) * 1e-3).astype(np.float32)
+    t_o, s_o = tables.copy(), state.copy()
+    uniq, seg, _ = O.embbag_bwd_adagrad(t_o, s_o, b.indices, b.offsets, cfg.B, gp, cfg.lr, cfg.eps)
+    t_g, s_g, uniq_g, seg_g, _, st = _bwd(cfg, b, tables, state, gp)
+    assert st == 0 and np.array_equal(uniq_g, uniq) and np.array_equal(seg_g, seg)
+    # a row's sum has up to 1040 terms, added in two levels of at most 65 and 16: 81 * 2^-24 = 5e-6 of their size
+    assert_close(t_g - tables, t_o.astype(np.float64) - tables, 3e-5, f"table update, {seed}")
+    assert_close(s_g, s_o, 2e-5, f"row state, {seed}")
 
 
 # bag lengths around the rounds of the gather, odd batches (the last block is not full)
