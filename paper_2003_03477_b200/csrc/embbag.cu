@@ -102,65 +102,147 @@ embbag_fwd_kernel(const float* __restrict__ tables, int T, uint32_t N, int D,
 // Rows of 65 to 256 floats, many bags: a block takes a stretch of consecutive bags, and the blocks that land on an SM at launch
 // take neighbouring stretches, so an SM stays with one table and finds its popular rows in L1; with half of the threads there
 // are enough registers for every row of a round to be in flight.  What bounds the form above there is the latency of rows from
-// L2, half of which another SM has just read as well.  us alone (L2 flushed), before -> now: 26 tables x 65 600 lookups of 128
-// floats 84 -> 74, 26 x 32 800 52 -> 45, 8 x 21 500 of 256 floats 33 -> 29.  1536 threads an SM at 40 registers: 121 and 68;
-// narrower rows gain nothing (64 floats 28.7 -> 30, 16 floats 45 -> 47), and beside other replicas' kernels they lose.
+// L2, half of which another SM has just read as well; narrower rows gain nothing (64 floats 28.7 -> 30 us, 16 floats 45 -> 47).
+// Nothing evens the blocks out once they run, so a stretch is cut by work, not by bags.  us in a row, form above / equal numbers of
+// bags / equal work, rows of 128 floats of 26 tables, batch 4096, ids of Zipf 1.05: 8 lookups a bag 55.6 / 41.9 / 43.4; one
+// table 40 and the others 2 30.8 / 112 / 23.4; one twice the others 59.5 / 70 / 48.8; 1 to 100 by table 79 / 269 / 55; one
+// lookup a bag 14.5 / 14.8 / 15.2 (batch 8191 34.6 / 36.0 / 30.7).  256 floats, 8 tables, batch 2048, 2 a bag: 6.3 / 8.7 / 8.0.
 constexpr int kStretchThreads = 512, kStretchBlocks = 2;   // blocks per SM
+constexpr uint32_t kBagWork = 3;                           // what a bag takes beside its lookups, in lookups (of 1 to 4)
+
+// Bags [first, end) of stretch k of `stretches`: a stretch begins at the first bag i with offsets[i] + kBagWork * i at or above k
+// equal shares of the whole.  Each half of the block looks for one end: among up to 1024 bags all at once, among more at 256
+// places first (one load after the other; 1.3 us).  Whatever the offsets hold, a larger share is not found earlier, and the
+// stretch before ends where this one begins: every bag is in one stretch.
+__device__ __forceinline__ void stretch_of(int k, int stretches, const int32_t* __restrict__ offsets, uint32_t bags, uint32_t& first,
+                                           uint32_t& end) {
+  constexpr uint32_t kHalf = kStretchThreads / 2, kEach = 4, kWarps = kHalf / 32;
+  __shared__ uint32_t s_below[2][2][kWarps], s_cut[2];
+  const uint32_t half = threadIdx.x / kHalf, at = threadIdx.x % kHalf, lane = threadIdx.x & 31;
+  const int32_t last = offsets[bags];
+  uint32_t lo = 0, hi = bags, step;                        // the place is in [lo, hi]
+  int round = 0;
+  do {
+    step = hi - lo > kEach * kHalf ? (hi - lo + kHalf - 1) / kHalf : 1u;
+    int32_t value[kEach];
+#pragma unroll
+    for (uint32_t u = 0; u < kEach; ++u) {
+      const uint32_t i = lo + (at + u * kHalf + 1) * step - 1;
+      value[u] = i < hi ? offsets[i] : 0;
+    }
+    const uint64_t want = (uint64_t)((uint32_t)max(last, 0) + kBagWork * bags) * (uint32_t)(k + half);   // `stretches` times as much
+    uint32_t below = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < kEach; ++u) {
+      if (lo + u * kHalf * step >= hi) break;              // (the same for all threads of the half)
+      const uint32_t i = lo + (at + u * kHalf + 1) * step - 1;
+      below += i < hi && (uint64_t)((uint32_t)max(value[u], 0) + kBagWork * i) * (uint32_t)stretches < want;
+    }
+    below = __reduce_add_sync(0xffffffffu, below);
+    if (lane == 0) s_below[round & 1][half][at >> 5] = below;
+    if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(kStretchThreads / 2) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(kStretchThreads / 2) : "memory");
+    below = __reduce_add_sync(0xffffffffu, lane < kWarps ? s_below[round & 1][half][lane] : 0u);
+    lo += below * step;
+    hi = min(hi, lo + step - 1);
+    ++round;
+  } while (step > 1);
+  if (at == 0) s_cut[half] = lo;
+  __syncthreads();
+  first = k > 0 ? s_cut[0] : 0u;
+  end = k + 1 < stretches ? s_cut[1] : bags;
+}
+
 template <int G>
 __global__ void __launch_bounds__(kStretchThreads, kStretchBlocks)
 embbag_fwd_stretch_kernel(const float* __restrict__ tables, int T, uint32_t N, int D,
                           const int32_t* __restrict__ indices, const int32_t* __restrict__ offsets, int B,
                           float* __restrict__ out_f32, int64_t ld_f32,
                           __nv_bfloat16* __restrict__ out_bf16, int64_t ld_bf16, int col0,
-                          int sms, int per_block, int32_t* __restrict__ d_status) {
+                          int sms, int32_t* __restrict__ d_status) {
   wait_for_previous_kernel();
   constexpr int kGroups = kStretchThreads / G, NV = 2, kRows = 4;
   const int grp = threadIdx.x / G, lane = threadIdx.x % G;
-  const int64_t bags = (int64_t)T * B;
-  const int64_t first = (int64_t)((int)blockIdx.x % sms * kStretchBlocks + (int)blockIdx.x / sms) * per_block;
-  const int64_t end = min(bags, first + per_block);
-  if (first >= end) return;
+  const uint32_t bags = (uint32_t)T * (uint32_t)B;
+  uint32_t first, end;
+  stretch_of((int)blockIdx.x % sms * kStretchBlocks + (int)blockIdx.x / sms, sms * kStretchBlocks, offsets, bags, first, end);
   const int L = __ldg(offsets + bags);
   const uint32_t nvec = (uint32_t)D >> 2;
-  int t = (int)(first / B), b = (int)(first - (int64_t)t * B) + grp, bad = 0;
-  for (int64_t i = first + grp; i < end; i += kGroups, b += kGroups) {
-    while (b >= B) { b -= B; ++t; }
-    int lo = offsets[i], hi = offsets[i + 1];
-    if (lo < 0 || hi < lo || hi > L) { bad |= SS_DEV_BAD_OFFSET; lo = hi = 0; }   // as above: an empty bag
-    const float4* tab = reinterpret_cast<const float4*>(tables + (int64_t)t * N * D);
-    float4 acc[NV];
+  int t = (int)(first / (uint32_t)B), b = (int)(first % (uint32_t)B) + grp, bad = 0;
+  // A lane group's bags of the stretch, P of them side by side.  (The round is written out: as a function that the other form
+  // shares, the compiler makes 10 % more of it here, 43.4 -> 47 to 49 us.)
+  auto sum_bags = [&](auto bags_at_once) {
+    constexpr int P = decltype(bags_at_once)::value, kEach = kRows / P;
+    for (uint32_t i = first + grp; i < end; i += P * kGroups, b += P * kGroups) {
+      while (b >= B) { b -= B; ++t; }
+      int lo[P], hi[P];
+      float4 acc[P][NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int j = lo; j < hi; j += kRows) {
-      uint32_t idx[kRows];
+      for (int p = 0; p < P; ++p) {
+        lo[p] = hi[p] = 0;
+        if (p == 0 || i + p * kGroups < end) {
+          lo[p] = offsets[i + p * kGroups];
+          hi[p] = offsets[i + p * kGroups + 1];
+        }
 #pragma unroll
-      for (int u = 0; u < kRows; ++u) idx[u] = (j + u < hi) ? (uint32_t)__ldg(indices + j + u) : 0xffffffffu;
-      float4 rowv[kRows][NV];
+        for (int v = 0; v < NV; ++v) acc[p][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      const float4* tab[P];
+      int tp[P], bp[P];
 #pragma unroll
-      for (int u = 0; u < kRows; ++u) {
-        const bool ok = idx[u] < N;
-        if (!ok && j + u < hi) bad |= SS_DEV_BAD_INDEX;
+      for (int p = 0; p < P; ++p) {
+        tp[p] = t; bp[p] = b + p * kGroups;
+        while (p > 0 && bp[p] >= B) { bp[p] -= B; ++tp[p]; }
+        tab[p] = reinterpret_cast<const float4*>(tables + (int64_t)tp[p] * N * D);
+        if (lo[p] < 0 || hi[p] < lo[p] || hi[p] > L) { bad |= SS_DEV_BAD_OFFSET; lo[p] = hi[p] = 0; }   // as above: an empty bag
+      }
+      while (lo[0] < hi[0] || (P > 1 && lo[P - 1] < hi[P - 1])) {
+        uint32_t idx[P][kEach];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const uint32_t c = lane + v * G;
-          rowv[u][v] = (ok && c < nvec) ? __ldg(tab + (idx[u] * nvec + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) idx[p][u] = (lo[p] + u < hi[p]) ? (uint32_t)__ldg(indices + lo[p] + u) : 0xffffffffu;
+        float4 rowv[P][kEach][NV];
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) {
+            const bool ok = idx[p][u] < N;
+            if (!ok && lo[p] + u < hi[p]) bad |= SS_DEV_BAD_INDEX;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+              const uint32_t c = lane + v * G;
+              rowv[p][u][v] = (ok && c < nvec) ? __ldg(tab[p] + (idx[p][u] * nvec + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+#pragma unroll
+          for (int u = 0; u < kEach; ++u)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[p][v] = add4(acc[p][v], rowv[p][u][v]);
+          lo[p] += kEach;
         }
       }
 #pragma unroll
-      for (int u = 0; u < kRows; ++u)
+      for (int p = 0; p < P; ++p) {
+        if (p > 0 && i + p * kGroups >= end) break;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) acc[v] = add4(acc[v], rowv[u][v]);
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int c = lane + v * G;
-      if (c < (int)nvec) {
-        const int64_t col = (int64_t)col0 + (int64_t)t * D + 4 * c;
-        if (out_f32) *reinterpret_cast<float4*>(out_f32 + (int64_t)b * ld_f32 + col) = acc[v];
-        if (out_bf16) *reinterpret_cast<uint2*>(out_bf16 + (int64_t)b * ld_bf16 + col) = bf16x4(acc[v]);
+        for (int v = 0; v < NV; ++v) {
+          const int c = lane + v * G;
+          if (c < (int)nvec) {
+            const int64_t col = (int64_t)col0 + (int64_t)tp[p] * D + 4 * c;
+            if (out_f32) *reinterpret_cast<float4*>(out_f32 + (int64_t)bp[p] * ld_f32 + col) = acc[p][v];
+            if (out_bf16) *reinterpret_cast<uint2*>(out_bf16 + (int64_t)bp[p] * ld_bf16 + col) = bf16x4(acc[p][v]);
+          }
+        }
       }
     }
-  }
+  };
+  if (first >= end) return;
+  // short bags: the latency of a bag's offsets, indices and rows is all there is (one lookup a bag: 16.4 -> 15.2 us, 37 -> 31)
+  if (max(offsets[end], 0) - max(offsets[first], 0) <= 2 * (int64_t)(end - first)) sum_bags(std::integral_constant<int, 2>());
+  else sum_bags(std::integral_constant<int, 1>());
   if (bad && d_status) atomicOr(d_status, bad);
 }
 
@@ -172,12 +254,13 @@ static void launch_fwd(const float* tables, int T, int64_t N, int D, const int32
   // for narrower rows the single-float4 form is the faster one)
   constexpr int FG = (NV == 1 && G == 32) ? 16 : G, FNV = (NV == 1 && G == 32) ? 2 : NV;
   if constexpr (FNV == 2) {
-    // from the point on where the bags fill every SM once, two of them or more for a lane group of a stretch
-    const int64_t bags = (int64_t)T * B, grid = (int64_t)num_sms() * kStretchBlocks;
-    if (bags * FG >= 2048ll * num_sms()) {
+    // from the point on where the bags fill every SM once, two of them or more for a lane group of a stretch (and up to where
+    // the work of all of them fits 32 bits)
+    const int64_t bags = (int64_t)T * B;
+    if (bags * FG >= 2048ll * num_sms() && bags < (1ll << 28)) {
       SS_TIMED("embbag_fwd_kernel", st);
-      launch_dependent(embbag_fwd_stretch_kernel<FG>, (unsigned)grid, kStretchThreads, 0, st, tables, T, (uint32_t)N, D, indices, offsets,
-                       B, out_f32, ld_f32, out_bf16, ld_bf16, col0, num_sms(), (int)((bags + grid - 1) / grid), d_status);
+      launch_dependent(embbag_fwd_stretch_kernel<FG>, (unsigned)(num_sms() * kStretchBlocks), kStretchThreads, 0, st, tables, T,
+                       (uint32_t)N, D, indices, offsets, B, out_f32, ld_f32, out_bf16, ld_bf16, col0, num_sms(), d_status);
       return;
     }
   }

@@ -355,3 +355,79 @@ def test_fwd_stretches_of_bags_match_the_sum_of_their_rows(D, T):
     same = torch.ones(T * B, dtype=torch.bool, device="cuda")
     same[[bad_bag, cut, cut + 1]] = False
     assert torch.equal(again[same], got[same])
+
+
+def _csr_batch(lens, N, D, T, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    off = torch.zeros(lens.numel() + 1, dtype=torch.int64, device="cuda")
+    torch.cumsum(lens, 0, out=off[1:])
+    idx = torch.randint(0, N, (int(off[-1]),), generator=g, device="cuda")
+    return torch.randn(T, N, D, generator=g, device="cuda"), idx, off
+
+
+def _uneven(kind, T, B, g):
+    """Bag lengths of T tables that differ in them."""
+    t = torch.arange(T, device="cuda").view(T, 1).expand(T, B)
+    r = torch.rand(T, B, generator=g, device="cuda")
+    lens = {"one_long": torch.where(t == T // 2, 40, 2), "first_long": torch.where(t == 0, 40, 1), "last_long": torch.where(t == T - 1, 40, 0),
+            "halves": torch.where(t < T // 2, 1, 9), "by_table": t % 23, "one_lookup": torch.ones_like(t), "one_bag": (r == r.max()) * 60_000,
+            "few_long_bags": torch.where(r < 0.01, 100, (r * 3).long()), "empty": torch.zeros_like(t)}[kind]
+    return lens.reshape(-1).long()
+
+
+# the same form where tables differ in bag length: its stretches are cut by work, short bags are summed two at a time
+@pytest.mark.parametrize("kind", ["one_long", "first_long", "last_long", "halves", "by_table", "one_lookup", "one_bag", "few_long_bags", "empty"])
+@pytest.mark.parametrize("D,T", [(128, 7), (100, 300), (256, 3)])
+def test_fwd_stretches_of_uneven_tables(D, T, kind):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = sms * 2048 // (16 if D <= 128 else 32) // T + 3
+    N = 61
+    lens = _uneven(kind, T, B, torch.Generator(device="cuda").manual_seed(D))
+    tables, idx, off = _csr_batch(lens, N, D, T, D)
+    table = torch.repeat_interleave(torch.arange(T * B, device="cuda") // B, lens)
+    want = torch.nn.functional.embedding_bag(idx + table * N, tables.double().view(T * N, D), off, mode="sum", include_last_offset=True)
+    i32, o32, st = torch.cat([idx, idx[:1], torch.zeros(1, dtype=idx.dtype, device="cuda")])[:max(idx.numel(), 1)].int(), off.int(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.full((B, T * D), -7.0, device="cuda")
+    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D, None, 0, 0, st)
+    got = out.view(B, T, D).transpose(0, 1).reshape(T * B, D).double()
+    assert int(st.item()) == 0
+    # n terms of size up to 5 added in float: n * 2^-24 of 5 n at most; sums of n random terms stay far below that bound
+    n = lens.max().clamp(min=1).double()
+    assert float((got - want).abs().max()) <= float(n * 2.0 ** -24 * 5 * n.sqrt() * 4)
+    # offsets that ascend nowhere near everywhere: every bag is written all the same, the sound ones with their sums
+    g = torch.Generator(device="cuda").manual_seed(1)
+    at = torch.randint(0, T * B, (max(T * B // 3, 1),), generator=g, device="cuda")
+    o32[at] = torch.randint(-2 ** 31, 2 ** 31 - 1, at.shape, generator=g, device="cuda").int()
+    out.fill_(-7.0)
+    st.zero_()
+    ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, out, T * D, None, 0, 0, st)
+    again = out.view(B, T, D).transpose(0, 1).reshape(T * B, D).double()
+    lo, hi, L = o32[:-1].long(), o32[1:].long(), int(off[-1])
+    same = (lo == off[:-1]) & (hi == off[1:])
+    empty = (lo < 0) | (hi < lo) | (hi > L)
+    assert int(st.item()) & ss.SS_DEV_BAD_OFFSET and torch.equal(again[same], got[same]) and not bool(again[empty].any())
+
+
+# the lookup's time follows its lookups, not which table they are in: an even batch and one with a table 20 times as long as the
+# others take about the same for the same number of lookups (with blocks that take equal numbers of bags: 4.5 times)
+def test_fwd_of_one_long_table_is_as_fast_as_of_even_ones():
+    T, B, D, N = 26, 4096, 128, 100_000
+    even, uneven = torch.full((T, B), 3, device="cuda"), torch.full((T, B), 2, device="cuda")
+    even[:12] = 4
+    uneven[T // 3] = 40
+    us = []
+    for lens in (even, uneven):
+        tables, idx, off = _csr_batch(lens.reshape(-1), N, D, T, 5)
+        i32, o32, st = idx.int(), off.int(), torch.zeros(1, dtype=torch.int32, device="cuda")
+        out = torch.empty(B, T * D, dtype=torch.bfloat16, device="cuda")
+        times = []
+        for _ in range(20):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, None, 0, out, T * D, 0, st)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        us.append(min(times))
+    assert us[1] <= 2 * us[0], us
