@@ -1483,19 +1483,13 @@ struct LaneColumns {
   __device__ __forceinline__ uint32_t next(int v) const { return inside(v) ? 16u * v * G : 0u; }   // beyond first()
 };
 
-// Sum over the group of g^2, the same in every lane.  The lanes' parts are added in the order of a tree over 2 * G lanes (H = 2)
-// or G lanes (H = 1): with H = 2 a lane holds what two lanes G apart would hold.
-template <int G, int NV, int H>
+// Sum over the group of g^2, the same in every lane: a lane's own columns first, then a tree over the lanes.
+template <int G, int NV>
 __device__ __forceinline__ float square_sum(const float4 (&g)[NV], unsigned mask) {
-  float part[H];
+  float ss = 0.f;
 #pragma unroll
-  for (int h = 0; h < H; ++h) {
-    part[h] = 0.f;
-#pragma unroll
-    for (int v = h; v < NV; v += H)
-      part[h] += __fmaf_rn(g[v].w, g[v].w, __fmaf_rn(g[v].z, g[v].z, __fmaf_rn(g[v].x, g[v].x, __fmul_rn(g[v].y, g[v].y))));
-  }
-  float ss = H == 2 ? part[0] + part[H - 1] : part[0];
+  for (int v = 0; v < NV; ++v)
+    ss += __fmaf_rn(g[v].w, g[v].w, __fmaf_rn(g[v].z, g[v].z, __fmaf_rn(g[v].x, g[v].x, __fmul_rn(g[v].y, g[v].y))));
 #pragma unroll
   for (int off = G / 2; off >= 1; off >>= 1) ss += __shfl_xor_sync(mask, ss, off, G);
   return ss;
@@ -1522,7 +1516,7 @@ __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t k
 #pragma unroll
   for (int v = 0; v < NV; ++v) r[v] = (lane + v * G < nvec) ? row[lane + v * G] : make_float4(0.f, 0.f, 0.f, 0.f);
   const float st = row_state[key];
-  const float ss = square_sum<G, NV, 1>(g, gmask);
+  const float ss = square_sum<G, NV>(g, gmask);
   const float sn = next_state<Wide>(st, ss, D), scale = step_scale<Wide>(lr, sn, eps);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -1536,7 +1530,7 @@ __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t k
   if (lane == 0) row_state[key] = sn;
 }
 
-template <int G, int NV, int H, int KB, int kMinBlocks, bool Exact, bool Wide>
+template <int G, int NV, int KB, int kMinBlocks, bool Exact, bool Wide>
 __global__ void __launch_bounds__(kWaThreads, kMinBlocks)
 window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
                     const int32_t* __restrict__ uidx, int L, uint32_t sentinel, int T, uint32_t N, int D, int B,
@@ -1617,7 +1611,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
     float4 f[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) f[v] = col.inside(v) ? floats_of(g[v]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float ss = square_sum<G, NV, H>(f, kAll);
+    const float ss = square_sum<G, NV>(f, kAll);
     const float sn = next_state<Wide>(st, ss, D), scale = -step_scale<Wide>(lr, sn, eps);
     const uint64_t s2 = (uint64_t)__float_as_uint(scale) << 32 | __float_as_uint(scale);
     __syncwarp();                                          // every lane has read the state
@@ -1914,20 +1908,20 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
   adagrad_row_nv<G, NV, true>(g, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
 }
 
-// Lanes a window, float4 a lane, halves of the sum-of-squares tree, positions a batch and blocks per SM (of 128 threads: 8 leave
+// Lanes a window, float4 a lane, positions a batch and blocks per SM (of 128 threads: 8 leave
 // a thread 64 registers, 10 leave 48).  A request should cover 128 bytes of a row: groups of 4 lanes with 4 float4 each move rows
 // of 256 bytes at half the rate (random rows of 7 GB: 8.7 G a second, groups of 8 or 16 15.9 G).  More warps beat more requests
 // a warp: 16 float4 in flight a lane, at 120 registers, took 62 us where 8, at 64, take 51.
-template <int G_, int NV_, int H_, int KB_, int kMinBlocks_> struct WindowShape {
-  static constexpr int G = G_, NV = NV_, H = H_, KB = KB_, kMinBlocks = kMinBlocks_;
+template <int G_, int NV_, int KB_, int kMinBlocks_> struct WindowShape {
+  static constexpr int G = G_, NV = NV_, KB = KB_, kMinBlocks = kMinBlocks_;
 };
 // by the float4 a row has, rounded up to a power of two (us of the reduction half, before -> now)
 template <int kQuads> struct WindowShapeFor;
-template <> struct WindowShapeFor<4> { using type = WindowShape<4, 1, 1, 4, 7>; };     // 40 x 32 900 lookups of 16 floats: 104 -> 91
-template <> struct WindowShapeFor<8> { using type = WindowShape<8, 1, 1, 2, 10>; };    // 16 x 43 000 of 32: 42 -> 37
-template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 1, 2, 8>; };    // 26 x 21 500 of 64: 58 -> 51
-template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
-template <> struct WindowShapeFor<64> { using type = WindowShape<32, 2, 1, 2, 6>; };   // 8 x 21 500 of 256: 68 -> 51; 5 x 9 000 of 200: 20 -> 20
+template <> struct WindowShapeFor<4> { using type = WindowShape<4, 1, 4, 7>; };     // 40 x 32 900 lookups of 16 floats: 104 -> 91
+template <> struct WindowShapeFor<8> { using type = WindowShape<8, 1, 2, 10>; };    // 16 x 43 000 of 32: 42 -> 37
+template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 2, 8>; };    // 26 x 21 500 of 64: 58 -> 51
+template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
+template <> struct WindowShapeFor<64> { using type = WindowShape<32, 2, 2, 6>; };   // 8 x 21 500 of 256: 68 -> 51; 5 x 9 000 of 200: 20 -> 20
 
 template <int G, int NV, bool kFuse>
 static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
@@ -1955,8 +1949,8 @@ static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, i
                          reinterpret_cast<int32_t*>(ws + p.off_uidx), (int)p.L, sentinel, T, (uint32_t)N, D, B, grad, ld_grad, col0,
                          partial, long_list, scalars, p.nwin, d_status, tables, row_state, lr, eps);
       };
-      if (D == S::G * S::NV * 4) go(window_apply_kernel<S::G, S::NV, S::H, S::KB, S::kMinBlocks, true, kWide>);
-      else go(window_apply_kernel<S::G, S::NV, S::H, S::KB, S::kMinBlocks, false, kWide>);
+      if (D == S::G * S::NV * 4) go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, true, kWide>);
+      else go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, false, kWide>);
     };
     window(typename WindowShapeFor<G * NV>::type());
   } else {
