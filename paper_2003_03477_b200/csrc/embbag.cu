@@ -1530,7 +1530,7 @@ __device__ __forceinline__ void adagrad_row_nv(const float4 (&g)[NV], uint32_t k
   if (lane == 0) row_state[key] = sn;
 }
 
-template <int G, int NV, int KB, int kMinBlocks, bool Exact, bool Wide>
+template <int G, int NV, int KB, int kMinBlocks, int KR, bool Exact, bool Wide>
 __global__ void __launch_bounds__(kWaThreads, kMinBlocks)
 window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
                     const int32_t* __restrict__ uidx, int L, uint32_t sentinel, int T, uint32_t N, int D, int B,
@@ -1629,7 +1629,25 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = Quad{0ull, 0ull};
 #pragma unroll 1
-  for (int i0 = 0; i0 < kWin; i0 += KB) {
+  for (int i0 = 0; i0 < kWin;) {
+    if constexpr (KR > 0) {
+      // no run of the warp's windows ends in the next KR positions: no row is needed, and there is room for more gradients
+      if (i0 + KR <= kWin && !__any_sync(kAll, tm >> i0 & ((1u << KR) - 1u))) {
+        Quad gv[KR][NV];
+#pragma unroll
+        for (int u = 0; u < KR; ++u) {
+          const char* const p = gl + (int64_t)s_row[w0 + i0 + u] * 16;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) gv[u][v] = quad_nc(p + col.next(v));
+        }
+#pragma unroll
+        for (int u = 0; u < KR; ++u)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc[v] = add_quad(acc[v], gv[u][v]);
+        i0 += KR;
+        continue;
+      }
+    }
     Quad gv[KB][NV], rv[KB][NV];
     float st[KB];
     uint32_t key[KB];
@@ -1674,6 +1692,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
         }
       }
     }
+    i0 += KB;
   }
   // ---- a run that starts in this window and goes on: its parts are added here, in window order, if they are all of this
   // block and no more than kShortSpan; otherwise the row enters the combine kernel's list
@@ -1737,7 +1756,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
 template <int G, int NV, bool FUSE, bool Wide>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
-                    const int32_t* __restrict__ long_list, int nwin, int D, const float* __restrict__ partial,
+                    const int32_t* __restrict__ long_list, int nwin, int nb_long, int D, const float* __restrict__ partial,
                     float* __restrict__ gsum, int64_t L, uint32_t sentinel, int64_t umax,
                     const int32_t* __restrict__ uniq, float* __restrict__ tables, float* __restrict__ row_state,
                     float lr, float eps) {
@@ -1761,14 +1780,6 @@ combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
   // fastest (the call 66.7 us against 69.5 with 32 and 89.8 with 128).
   constexpr int kShort = kShortSpan;
   constexpr int kBatch = NV <= 1 ? 8 : (NV <= 2 ? 4 : 2);
-  // The two phases are two chains of dependent loads; with enough blocks the first part of the grid takes the long
-  // spans (phase B) and the rest the short ones (phase A), so that the chains run side by side instead of
-  // one after the other.  A small grid does both in every block.  Half of the grid for each where the window kernel leaves
-  // all crossing runs; behind the fused one few short spans are left, and most of 8 blocks per SM only took other kernels'
-  // places: with 5 per SM, a quarter of them for the short spans, four replicas of the ordinary model take 452 us a round
-  // instead of 455, three of an odd-sized one 104 instead of 106 (the call alone 51 and 51, 93 and 93 for 128 floats; 3 per SM:
-  // 449 and 103, but 54 and 100).
-  const int nb_long = gridDim.x >= 4 ? (FUSE ? (int)gridDim.x * 3 / 4 : (int)gridDim.x / 2) : 0;
   const bool do_short = nb_long == 0 || (int)blockIdx.x >= nb_long;
   const bool do_long = nb_long == 0 || (int)blockIdx.x < nb_long;
   const int a_blk = nb_long == 0 ? (int)blockIdx.x : (int)blockIdx.x - nb_long;
@@ -1908,20 +1919,43 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
   adagrad_row_nv<G, NV, true>(g, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
 }
 
-// Lanes a window, float4 a lane, positions a batch and blocks per SM (of 128 threads: 8 leave
-// a thread 64 registers, 10 leave 48).  A request should cover 128 bytes of a row: groups of 4 lanes with 4 float4 each move rows
-// of 256 bytes at half the rate (random rows of 7 GB: 8.7 G a second, groups of 8 or 16 15.9 G).  More warps beat more requests
-// a warp: 16 float4 in flight a lane, at 120 registers, took 62 us where 8, at 64, take 51.
-template <int G_, int NV_, int KB_, int kMinBlocks_> struct WindowShape {
-  static constexpr int G = G_, NV = NV_, KB = KB_, kMinBlocks = kMinBlocks_;
+// Lanes a window, float4 a lane, positions a batch, blocks per SM (of 128 threads: 8 leave a thread 64 registers, 10 leave 48),
+// positions at once where no run ends (0: as any others).  A request should cover 128 bytes of a row: groups of 4 lanes with 4
+// float4 each move rows of 256 bytes at half the rate (random rows of 7 GB: 8.7 G a second, groups of 8 or 16 15.9 G).  More warps
+// beat more requests a warp: 16 float4 in flight a lane, at 120 registers, took 62 us where 8, at 64, take 51.
+template <int G_, int NV_, int KB_, int kMinBlocks_, int KR_> struct WindowShape {
+  static constexpr int G = G_, NV = NV_, KB = KB_, kMinBlocks = kMinBlocks_, KR = KR_;
 };
-// by the float4 a row has, rounded up to a power of two (us of the reduction half, before -> now)
+// By the float4 a row has, rounded up to a power of two.  `few` is for up to kFew windows per SM, about as many as its blocks hold
+// at once: then a window's own rounds are all the time there is, and more lanes or more registers for them are what counts.
+// us of the update half, 26 tables (of 256 floats 10), as it was with `few` throughout (128 floats: one position a batch at 48
+// registers, which spilled) -> now, for 20 000 lookups a table hit once / 66 / 200 times a row, and Zipf 1.2:
 template <int kQuads> struct WindowShapeFor;
-template <> struct WindowShapeFor<4> { using type = WindowShape<4, 1, 4, 7>; };     // 40 x 32 900 lookups of 16 floats: 104 -> 91
-template <> struct WindowShapeFor<8> { using type = WindowShape<8, 1, 2, 10>; };    // 16 x 43 000 of 32: 42 -> 37
-template <> struct WindowShapeFor<16> { using type = WindowShape<8, 2, 2, 8>; };    // 26 x 21 500 of 64: 58 -> 51
-template <> struct WindowShapeFor<32> { using type = WindowShape<16, 2, 1, 10>; };  // 26 x 32 800 of 128: 94 -> 93, 26 x 65 600: 168 -> 167
-template <> struct WindowShapeFor<64> { using type = WindowShape<32, 2, 2, 6>; };   // 8 x 21 500 of 256: 68 -> 51; 5 x 9 000 of 200: 20 -> 20
+template <> struct WindowShapeFor<4> {                     // 16 floats 19 / 14 / 20 / 32 (8 blocks 19 / 14 / 20 / 33)
+  static constexpr int kFew = 0;
+  using many = WindowShape<4, 1, 4, 7, 0>;
+  using few = many;
+};
+template <> struct WindowShapeFor<8> {                     // 32 floats 29 / 20 / 27 / 39 -> 24 / 17 / 22 / 38, 17 to 31 floats alike;
+  static constexpr int kFew = 120;                         // 4000 lookups a table `few` 15, `many` 17
+  using many = WindowShape<4, 2, 2, 8, 4>;
+  using few = WindowShape<8, 1, 2, 10, 0>;
+};
+template <> struct WindowShapeFor<16> {                    // 64 floats 47 / 22 / 29 / 55 -> 47 / 22 / 28 / 54, 48 floats 47 / 25 / 31 / 60 ->
+  static constexpr int kFew = 0;                           // 48 / 24 / 30 / 61
+  using many = WindowShape<8, 2, 2, 8, 8>;
+  using few = many;
+};
+template <> struct WindowShapeFor<32> {                    // 128 floats 87 / 37 / 39 / 89 -> 85 / 36 / 37 / 85, 100 floats
+  static constexpr int kFew = 0;                           // 92 / 40 / 41 / 101 -> 87 / 37 / 38 / 94
+  using many = WindowShape<16, 2, 2, 8, 4>;
+  using few = many;
+};
+template <> struct WindowShapeFor<64> {                    // 256 floats 67 / - / - / 77 -> 65 / - / - / 72, 160 floats 63 / - / - / 73 ->
+  static constexpr int kFew = 28;                          // 57 / - / - / 65; 20 windows an SM `few` 17 to 20, `many` 18 to 22
+  using many = WindowShape<32, 2, 2, 8, 4>;
+  using few = WindowShape<32, 2, 2, 6, 0>;
+};
 
 template <int G, int NV, bool kFuse>
 static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
@@ -1949,10 +1983,12 @@ static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, i
                          reinterpret_cast<int32_t*>(ws + p.off_uidx), (int)p.L, sentinel, T, (uint32_t)N, D, B, grad, ld_grad, col0,
                          partial, long_list, scalars, p.nwin, d_status, tables, row_state, lr, eps);
       };
-      if (D == S::G * S::NV * 4) go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, true, kWide>);
-      else go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, false, kWide>);
+      if (D == S::G * S::NV * 4) go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, S::KR, true, kWide>);
+      else go(window_apply_kernel<S::G, S::NV, S::KB, S::kMinBlocks, S::KR, false, kWide>);
     };
-    window(typename WindowShapeFor<G * NV>::type());
+    using Shapes = WindowShapeFor<G * NV>;
+    if (p.nwin > Shapes::kFew * num_sms()) window(typename Shapes::many());
+    else if constexpr (Shapes::kFew > 0) window(typename Shapes::few());
   } else {
     SS_TIMED("window_reduce_kernel", st);
     launch_dependent(window_reduce_kernel<G, NV>, blocks, 256, 0, st, 
@@ -1961,11 +1997,20 @@ static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, i
   }
   {
     SS_TIMED("combine_rows_kernel", st);
-    const int per_sm = kFuse ? 5 : 8, cblocks = p.nwin < num_sms() * per_sm ? p.nwin : num_sms() * per_sm;
+    // The long spans and the short ones are two chains of dependent loads: with enough blocks the first part of the grid takes the
+    // long ones and the rest the short ones, so that the chains run side by side.  Half of 8 blocks per SM for each where the
+    // window kernel leaves all crossing runs, or leaves its block at every fourth window (wide rows; with a quarter of 5 per SM for
+    // the short spans 16 us instead of 14 where rows are looked up 66 times).  Behind the others few short spans are left, and most
+    // of 8 per SM only took other kernels' places: with 5, a quarter of them for the short spans, four replicas of the ordinary
+    // model take 452 us a round instead of 455, three of an odd-sized one 104 instead of 106 (the call alone 51 and 51, 93 and 93
+    // for 128 floats; 3 per SM: 449 and 103, but 54 and 100).
+    const bool few_short = kFuse && (!kWide || p.nwin <= WindowShapeFor<64>::kFew * num_sms());
+    const int per_sm = few_short ? 5 : 8, cblocks = p.nwin < num_sms() * per_sm ? p.nwin : num_sms() * per_sm;
+    const int long_blocks = cblocks < 4 ? 0 : few_short ? cblocks * 3 / 4 : cblocks / 2;   // 0: every block does both
     // fused rows of at least eight float4: two float4 per lane, half as many lanes per row, twice as many rows in flight
     constexpr int CG = (kFuse && !kWide && G >= 8) ? G / 2 : G, CNV = (kFuse && G >= 8) ? 2 : NV;
     launch_dependent(combine_rows_kernel<CG, CNV, kFuse, kWide>, cblocks, 256, (size_t)(256 / CG) * D * 4, st, 
-        seg, scalars, long_list, p.nwin, D, partial, gsum, p.L, sentinel, (int64_t)umax, uniq, tables, row_state, lr, eps);
+        seg, scalars, long_list, p.nwin, long_blocks, D, partial, gsum, p.L, sentinel, (int64_t)umax, uniq, tables, row_state, lr, eps);
   }
   if constexpr (!kFuse) {
     // every distinct row is updated from its sum in gsum

@@ -248,9 +248,9 @@ def test_apply_refuses_a_workspace_sorted_for_another_problem():
     assert int(st.item()) == 0 and not np.array_equal(dt.cpu().numpy(), tables)
 
 
-def _run_lengths_batch(D, lengths, B, seed):
+def _run_lengths_batch(D, lengths, B, seed, spare=0):
     """Two tables whose rows are looked up `lengths` times each, cut into B bags at random places (some are empty)."""
-    T, N = 2, len(lengths) + 3
+    T, N = 2, len(lengths) + 3 + spare
     cfg = synth.scaled(synth.CONFIGS["tiny"], T=T, N=N, D=D, B=B, bottom=(13, 64, D), top=(3 * D, 64, 1))
     rng = np.random.default_rng(seed)
     idx, off = [], [0]
@@ -272,20 +272,35 @@ def test_bwd_runs_around_windows_blocks_and_spans(D):
         _check_runs(D, extra + RUN_LENGTHS, seed)
 
 
-# rows of 129 to 256 floats once more with as many windows as the fused kernel wants (16 an SM)
-@pytest.mark.parametrize("D", [132, 200, 256])
-def test_bwd_runs_of_wide_rows_with_many_windows(D):
+# the same with as many windows per SM as the fused kernel wants of rows of 129 to 256 floats, and as its forms for many windows
+# want; rows that nobody looks up keep the lookups per row low enough for the fused kernel
+@pytest.mark.parametrize("D,per_sm,spare", [(132, 16, True), (200, 16, True), (256, 16, True), (132, 29, True), (256, 29, True),
+                                            (132, 16, False), (256, 29, False), (20, 121, False), (32, 121, False)])
+def test_bwd_runs_with_many_windows(D, per_sm, spare):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    repeats = -(-16 * sms * 16 // (2 * sum(RUN_LENGTHS))) + 1
-    _check_runs(D, [5] + RUN_LENGTHS * repeats, 4)
+    lengths = [5] + RUN_LENGTHS * (-(-per_sm * sms * 16 // (2 * sum(RUN_LENGTHS))) + 1)
+    _check_runs(D, lengths, 4, sum(lengths) // 32 if spare else 0)
+
+
+def _best_us(call):
+    times = []
+    for _ in range(20):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            call()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b) * 100)
+    return min(times)
 
 
 RUN_LENGTHS = [15, 1, 16, 16, 32, 17, 128, 1, 127, 2, 144, 7, 113, 1, 129, 3, 1, 1, 1, 260, 12, 33, 111, 1, 5, 600, 31, 96,
                97, 1, 14, 16, 48, 2, 1, 1, 1040, 30, 18, 112, 113]
 
 
-def _check_runs(D, lengths, seed):
-    cfg, b = _run_lengths_batch(D, lengths, 61, seed)
+def _check_runs(D, lengths, seed, spare=0):
+    cfg, b = _run_lengths_batch(D, lengths, 61, seed, spare)
     rng = np.random.default_rng(seed)
     tables = (rng.normal(size=(cfg.T, cfg.N, D)) * 0.05).astype(np.float32)
     state = (rng.random((cfg.T, cfg.N)) * 1e-4).astype(np.float32)
@@ -420,14 +435,5 @@ def test_fwd_of_one_long_table_is_as_fast_as_of_even_ones():
         tables, idx, off = _csr_batch(lens.reshape(-1), N, D, T, 5)
         i32, o32, st = idx.int(), off.int(), torch.zeros(1, dtype=torch.int32, device="cuda")
         out = torch.empty(B, T * D, dtype=torch.bfloat16, device="cuda")
-        times = []
-        for _ in range(20):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            for _ in range(10):
-                ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, None, 0, out, T * D, 0, st)
-            b.record()
-            b.synchronize()
-            times.append(a.elapsed_time(b) * 100)
-        us.append(min(times))
+        us.append(_best_us(lambda: ss.ss_embbag_fwd(tables, T, N, D, i32, o32, B, None, 0, out, T * D, 0, st)))
     assert us[1] <= 2 * us[0], us
