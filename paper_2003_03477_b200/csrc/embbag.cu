@@ -2022,12 +2022,22 @@ static void launch_reduce_as(const BwdPlan& p, char* ws, const uint32_t* keys, i
   }
 }
 
-// Rows of up to 128 floats are updated from the window kernel, wider ones than 256 from their sums in memory; in between it
-// depends on how many windows there are: a lane group of the fused kernel works through its 16 positions in eight dependent
-// rounds, which takes the time where the windows are few (lookup and update of 26 tables x 90 lookups of 248 floats: fused 34 us,
-// not fused 31), while the sums' way through memory does where they fill the SMs (8 x 21 500 of 256 floats 51 and 68 us, the
-// update alone; 5 x 9000 of 200, 19 windows an SM, 20 and 20).
-constexpr int kFuseWindows = 16;                           // per SM
+// Rows of up to 128 floats are updated from the window kernel, wider ones than 256 from their sums in memory.  In between the sums'
+// way through memory and back is what the fused kernel saves, a chain of dependent rounds for the 16 positions of a window what it
+// costs; so it needs windows enough to fill the SMs and rows that are not all popular (lookups per row of the tables: at least that
+// many a row on average, whichever rows they are).  us of the update half, fused / not:
+//   windows per SM      uniform ids, 132 / 192 / 256 floats        Zipf 1.05
+//   8                   17 / 15, 17 / 16, 16 / 16                  18 / 13, 18 / 13, 17 / 14
+//   16                  18 / 18, 20 / 20, 18 / 25                  19 / 16, 20 / 17, 18 / 18
+//   20                  18 / 21, 19 / 25, 18 / 34                  19 / 18, 18 / 18, 17 / 20
+//   32                  25 / 32, 26 / 40, 25 / 49                  26 / 24, 25 / 25, 22 / 27
+//   64                  42 / 61, 50 / 75, 54 / 84                  33 / 37, 36 / 43, 37 / 50
+//   lookups per row     (135 windows per SM for 132 floats, 90 for 160 to 256; 132 / 160 / 256 floats)
+//   25                  29 / 27, 27 / 28, 28 / 30
+//   66                  30 / 24, 29 / 24, 30 / 26
+//   200                 26 / 24, 24 / 23, 25 / 25
+//   4000                29 / 28, 28 / 29, 27 / 28
+constexpr int kFuseWindows = 16, kFuseHits = 32;           // per SM; per row
 template <int G, int NV>
 static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int T, int64_t N,
                           int D, int B, const float* grad, int64_t ld_grad, int col0, float* tables,
@@ -2037,7 +2047,7 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   };
   if constexpr (NV == 1) as(std::true_type());
   else if constexpr (NV > 2) as(std::false_type());
-  else if (p.nwin >= kFuseWindows * num_sms()) as(std::true_type());
+  else if (p.nwin >= kFuseWindows * num_sms() && p.L <= kFuseHits * T * N) as(std::true_type());
   else as(std::false_type());
 }
 

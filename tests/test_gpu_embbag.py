@@ -282,6 +282,19 @@ def test_bwd_runs_with_many_windows(D, per_sm, spare):
     _check_runs(D, lengths, 4, sum(lengths) // 32 if spare else 0)
 
 
+def _update_us(T, N, D, lookups, bag):
+    """us of the update half for T tables of N rows, all about equally often looked up."""
+    B = lookups // bag
+    g = torch.Generator(device="cuda").manual_seed(1)
+    off = torch.arange(0, T * B * bag + 1, bag, device="cuda").int()
+    idx = torch.randint(0, N, (T * B * bag,), generator=g, device="cuda").int()
+    tables, state = torch.zeros(T, N, D, device="cuda"), torch.ones(T * N, device="cuda")
+    grad, st = torch.randn(B, T * D, generator=g, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(ss.ss_embbag_bwd_workspace_bytes(T, N, D, B, idx.numel()), dtype=torch.uint8, device="cuda")
+    ss.ss_embbag_bwd_sort(T, N, D, idx, off, B, idx.numel(), ws, None, None, None, None, st)
+    return _best_us(lambda: ss.ss_embbag_bwd_apply(tables, state, T, N, D, B, idx.numel(), grad, T * D, 0, 0.01, 1e-8, ws, st))
+
+
 def _best_us(call):
     times = []
     for _ in range(20):
@@ -293,6 +306,12 @@ def _best_us(call):
         b.synchronize()
         times.append(a.elapsed_time(b) * 100)
     return min(times)
+
+
+# popular rows are summed, not updated lookup by lookup: what is left is reading the gradients.  Rows of 132 floats, 66 lookups of
+# each row against one: 0.66 of the time where the fused kernel took both, 0.45 now
+def test_bwd_of_popular_wide_rows_takes_the_time_of_their_gradients():
+    assert _update_us(12, 300, 132, 20_000, 10) <= 0.55 * _update_us(12, 20_000, 132, 20_000, 10)
 
 
 RUN_LENGTHS = [15, 1, 16, 16, 32, 17, 128, 1, 127, 2, 144, 7, 113, 1, 129, 3, 1, 1, 1, 260, 12, 33, 111, 1, 5, 600, 31, 96,
