@@ -1910,12 +1910,12 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
   const int64_t u = (int64_t)blockIdx.x * kGroups + grp;
   if (u >= min((int64_t)scalars[0], umax)) return;
   const uint32_t key = (uint32_t)uniq[u];
-  if (key >= sentinel) return;                             // never true for a consistent workspace
   const int nvec = D >> 2;
-  const float4* p = reinterpret_cast<const float4*>(gsum + u * D);
+  const float4* p = reinterpret_cast<const float4*>(gsum + u * D);   // on its way beside the key
   float4 g[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) g[v] = lane + v * G < nvec ? p[lane + v * G] : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (key >= sentinel) return;                             // never true for a consistent workspace
   adagrad_row_nv<G, NV, true>(g, key, lane, nvec, D, gmask, tables, row_state, lr, eps);
 }
 
