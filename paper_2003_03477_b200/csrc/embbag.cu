@@ -2071,18 +2071,23 @@ __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_f
 // few ranges as hold its lookups (four replicas of the ordinary model 478 us a round with two ranges a table, 494 with three).
 // Few tables are cut finer: down to 5500 lookups a range, while that takes no more than a quarter of the SMs, where the sort is
 // a call by itself, which runs beside other work (three replicas of 11 tables of 10 700 lookups 104 us a round; 107 with 2750 a
-// range, 121 with 1400 and half of the SMs); down to 1400, on half of them, where the update waits for the sort in the same call
-// (5 tables of 9000 lookups 26 -> 21.5 us, lookup and update 60 -> 55; 12 of 10 700 27 -> 22).  Blocks without a range cost
-// nothing that could be measured.
+// range, 121 with 1400 and half of the SMs); down to 1400, up to six ranges on a third of them, where the update waits for the sort
+// in the same call.  One such call alone would take half of the SMs (12 tables of 10 200 lookups: by the rule above 50 us, half 41,
+// a third 41; 20 of 6000 45 / 33 / 35), but several at a time lose more than that: three of 12 tables 62 / 61 / 54, four 72 / 80 / 68,
+// four of 11 64 / 73 / 63, four of 16 of 20 500 116 / 126 / 116.  With eight ranges a table's list is walked too often (3 of 32 800,
+// Zipf 1.2: 71 us, six 66), and two a table are still worth half of the SMs (26 of 5100: 42 us with one, 37).  Blocks without a
+// range cost nothing that could be measured.
 static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, bool waited_for, BucketSort* a, int64_t* blocks, int* nb) {
   const int64_t avg = (L + T - 1) / T;
   if (B > 65535 || avg > 44000) return false;              // bag numbers, plus one, take 16 bits
   int64_t C = (avg + kBsRange - 1) / kBsRange;
-  const int64_t least = waited_for ? 1400 : 5500, fine = (avg + least - 1) / least, room = num_sms() / (waited_for ? 2 : 4) / T;
+  const int64_t least = waited_for ? 1400 : 5500, fine = (avg + least - 1) / least, most = waited_for ? 6 : kBsMaxBuckets;
+  int64_t room = num_sms() / (waited_for ? 3 : 4) / T;
+  if (waited_for && room < 2) room = num_sms() / 2 / T;
   a->per_range = kBsRange;
   if (C < fine && C < room) {
     C = fine < room ? fine : room;
-    if (C > kBsMaxBuckets) C = kBsMaxBuckets;
+    if (C > most) C = most;
     a->per_range = (int)(avg * 115 / 100 / C);             // tables a little longer than the average get no further range
   }
   if (C < 1) C = 1;
