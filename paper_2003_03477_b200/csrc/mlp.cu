@@ -15,11 +15,15 @@ namespace ss {
 // One launch takes a list of such jobs.  A block owns 256 or 64 columns c and a slice of the batch; its 8
 // row groups add their rows in ascending order, the groups are added in order, and a second kernel
 // adds the slices in order: every sum has a fixed association.
-// What bounds it is the latency of a block's loads, so a thread keeps 8 rows (of 8 columns) or 16 rows (of two) in flight:
-// with 4 it took 13.8 / 34 us (the sums of the 2048- and the 4096-sample model), with 8 and 16 rows 8.5 / 28.  The first layer's
-// gradient takes two columns a thread (a row of S read from shared memory serves both; its loads start while the S tile is
-// filled) and all threads add the row groups: half as many blocks, of which three fit beside a tensor-core CTA.  28 -> 24 us for
-// the 4096-sample model, the same for the other, but four replicas of it take 455 us a round instead of 460.
+// What bounds it is the latency of a block's loads, so a thread keeps 8 rows (of 8 columns) or 16 rows (of one or two) in flight:
+// with 4 it took 13.8 / 34 us (the sums of the 2048- and the 4096-sample model), with 8 and 16 rows 8.5 / 28.  Where the first
+// layer's gradients are bf16, a thread takes two columns of them (a row of S read from shared memory serves both; its loads start
+// while the S tile is filled) and all threads add the row groups: half as many blocks, of which two fit beside a tensor-core CTA
+// (its 21 504 registers and theirs of 20 480).  28 -> 24 us for the 4096-sample model, the same for the other, but four replicas of
+// it take 455 us a round instead of 460.  Three blocks per SM leave a thread 80 registers, which costs 12 bytes of spills; without
+// them, the job's fields read from shared memory at each use, a pass takes 0.3 us more.  A block's job is found by one thread and
+// read from shared memory: read by every thread from the list itself, where only the kernel's parameters hold it, forward and
+// backward of 320-256-1 behind 13-512-64 took 57 us instead of 55 at 2048 samples.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMaxJobs = 2 * kMaxLayers + 2;
 constexpr int kMaxSCols = 16;
@@ -46,7 +50,6 @@ __device__ __forceinline__ float load_kind(const void* p, int kind, int64_t i) {
 
 constexpr int kRedRows = 256;     // most rows of the batch a block takes (bounds the staged S tile)
 constexpr int kRedWide = 256;     // columns per block of a job without a second factor matrix (s_cols = 1)
-constexpr int kRedPairs = 64;     // columns per block of a job with one
 
 // Eight consecutive elements M[row, c .. c+7] as floats; elements at or beyond ncols read as zero.  One
 // 128-bit load (bf16) or two (float) when the address allows it, element loads otherwise.
@@ -76,11 +79,11 @@ __device__ __forceinline__ void load8_kind(const void* p, int kind, int64_t row,
   }
 }
 
-// Rows ry, ry + 8, ... of two neighbouring columns, in ascending order, times the rows of S in s_tile: F rows in flight, the
+// Rows ry, ry + 8, ... of C neighbouring columns, in ascending order, times the rows of S in s_tile: F rows in flight, the
 // first ones while stage() fills s_tile.
-template <int F, typename Raw, typename Stage, typename Load, typename Value>
-__device__ __forceinline__ void two_column_sums(const float* s_tile, int ry, int nrows, float (&acc)[2][kMaxSCols], Stage stage, Load load,
-                                                Value value) {
+template <int C, int F, typename Raw, typename Stage, typename Load, typename Value>
+__device__ __forceinline__ void column_sums(const float* s_tile, int ry, int nrows, float2 (&acc)[C][kMaxSCols / 2], Stage stage, Load load,
+                                            Value value) {
   Raw m[F];
   auto fetch = [&](int rr) {
 #pragma unroll
@@ -93,22 +96,24 @@ __device__ __forceinline__ void two_column_sums(const float* s_tile, int ry, int
 #pragma unroll
     for (int u = 0; u < F; ++u) {
       if (rr + 8 * u >= nrows) break;
-      const float2 v = value(m[u]);
+      float v[C];
+      value(m[u], v);
       const float4* srow = reinterpret_cast<const float4*>(s_tile + (rr + 8 * u) * kMaxSCols);
 #pragma unroll
       for (int q4 = 0; q4 < kMaxSCols / 4; ++q4) {
         const float4 sv = srow[q4];                            // one 128-bit broadcast read for four columns of S
-        const float sq[4] = {sv.x, sv.y, sv.z, sv.w};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          acc[0][4 * q4 + k] = fmaf(v.x, sq[k], acc[0][4 * q4 + k]);
-          acc[1][4 * q4 + k] = fmaf(v.y, sq[k], acc[1][4 * q4 + k]);
+        for (int h = 0; h < C; ++h) {
+          acc[h][2 * q4] = fma2(make_float2(v[h], v[h]), make_float2(sv.x, sv.y), acc[h][2 * q4]);
+          acc[h][2 * q4 + 1] = fma2(make_float2(v[h], v[h]), make_float2(sv.z, sv.w), acc[h][2 * q4 + 1]);
         }
       }
     }
   }
 }
 
+// kCols: columns a thread takes of a job with a second factor matrix, 2 where that job's gradients are bf16
+template <int kCols>
 __global__ void __launch_bounds__(256, 3)
 batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int rows_per_split, float* __restrict__ partial) {
   wait_for_previous_kernel();
@@ -116,11 +121,15 @@ batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int row
   constexpr int kPartFloats = 8 * 32 * (kMaxSCols + 1);
   static_assert(kPartFloats >= kRedRows * kMaxSCols && kPartFloats >= 8 * kRedWide, "one buffer serves all three uses");
   __shared__ __align__(16) float s_tile[kPartFloats];
+  __shared__ RedJob s_job;
+  if (threadIdx.x == 0) {
+    int j = 0;
+    while (j + 1 < jobs.njobs && (int)blockIdx.x >= jobs.job[j + 1].tile0) ++j;
+    s_job = jobs.job[j];
+  }
+  __syncthreads();
+  const RedJob J = s_job;                                    // the job's fields in registers
   const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-  // the last job that begins at or before this column tile: every warp finds it by itself
-  int begun = 0;
-  for (int j = cx; j < jobs.njobs; j += 32) begun += (int)blockIdx.x >= jobs.job[j].tile0;
-  const RedJob J = jobs.job[__reduce_add_sync(0xffffffffu, begun) - 1];
   const int sc = J.s_cols;
   const int r0 = blockIdx.y * rows_per_split;
   const int r1 = min(B, r0 + rows_per_split);
@@ -203,12 +212,14 @@ batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int row
     return;
   }
 
-  // ---- a second factor with several columns (the layer with few inputs): 64 columns c per block, two neighbours a thread,
-  // which keeps one sum per column of S for each; a row of S read from shared memory serves both
-  const int c = ((int)blockIdx.x - J.tile0) * kRedPairs + 2 * cx;
-  float acc[2][kMaxSCols];
+  // ---- a second factor with several columns (the layer with few inputs): 32 or 64 columns c per block, one or two neighbours a
+  // thread, which keeps one sum per column of S for each; a row of S read from shared memory serves both
+  const int c0 = ((int)blockIdx.x - J.tile0) * 32 * kCols, c = c0 + kCols * cx;
+  float2 acc[kCols][kMaxSCols / 2];
 #pragma unroll
-  for (int q = 0; q < kMaxSCols; ++q) acc[0][q] = acc[1][q] = 0.f;
+  for (int h = 0; h < kCols; ++h)
+#pragma unroll
+    for (int q = 0; q < kMaxSCols / 2; ++q) acc[h][q] = make_float2(0.f, 0.f);
   auto stage = [&] {
     // S rows as float, padded with zeros to kMaxSCols columns so that the inner product needs no column test
     for (int i = threadIdx.x; i < nrows * kMaxSCols; i += 256) {
@@ -217,34 +228,30 @@ batch_reduce_partial_kernel(const __grid_constant__ RedJobs jobs, int B, int row
     }
     __syncthreads();
   };
-  if (J.m_kind == OP_BF16 && (J.ldm & 1) == 0 && (J.ncols & 1) == 0 && (reinterpret_cast<uintptr_t>(J.M) & 3u) == 0) {
+  if constexpr (kCols == 1) {
+    column_sums<1, 16, float>(
+        s_tile, ry, nrows, acc, stage,
+        [&](int r) { return c < J.ncols ? load_kind(J.M, J.m_kind, (int64_t)(r0 + r) * J.ldm + c) : 0.f; },
+        [](float m, float (&v)[1]) { v[0] = m; });
+  } else {                                                     // bf16, and a layer's width is a multiple of 8: pairs are whole and aligned
     const __nv_bfloat16* M = reinterpret_cast<const __nv_bfloat16*>(J.M) + (int64_t)r0 * J.ldm + c;
-    two_column_sums<16, uint32_t>(
+    column_sums<2, 16, uint32_t>(
         s_tile, ry, nrows, acc, stage,
         [&](int r) { return c < J.ncols ? *reinterpret_cast<const uint32_t*>(M + (int64_t)r * J.ldm) : 0u; },
-        [](uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); });   // a bf16 is the upper half of a float
-  } else {
-    two_column_sums<8, float2>(
-        s_tile, ry, nrows, acc, stage,
-        [&](int r) {
-          const int64_t i = (int64_t)(r0 + r) * J.ldm + c;
-          return make_float2(c < J.ncols ? load_kind(J.M, J.m_kind, i) : 0.f, c + 1 < J.ncols ? load_kind(J.M, J.m_kind, i + 1) : 0.f);
-        },
-        [](float2 v) { return v; });
+        [](uint32_t w, float (&v)[2]) { v[0] = __uint_as_float(w << 16); v[1] = __uint_as_float(w & 0xFFFF0000u); });   // a bf16 is the upper half of a float
   }
   __syncthreads();                                             // the S tile is no longer read
-  // the even columns of the block, then the odd ones: half the buffer, and a block fits beside a tensor-core CTA
+  // of two columns a thread the even ones first, then the odd ones, in the same buffer
   float (*part)[32][kMaxSCols + 1] = reinterpret_cast<float (*)[32][kMaxSCols + 1]>(s_tile);   // [8][32][17]
-  const int c0 = ((int)blockIdx.x - J.tile0) * kRedPairs;
   float* dst = partial + (int64_t)blockIdx.y * jobs.total + J.part_off;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < kCols; ++h) {
     if (h > 0) __syncthreads();
 #pragma unroll
-    for (int q = 0; q < kMaxSCols; ++q) part[ry][cx][q] = acc[h][q];
+    for (int q = 0; q < kMaxSCols; ++q) part[ry][cx][q] = q & 1 ? acc[h][q >> 1].y : acc[h][q >> 1].x;
     __syncthreads();
     for (int i = threadIdx.x; i < 32 * sc; i += 256) {
-      const int col = i / sc, q = i - col * sc, co = c0 + 2 * col + h;
+      const int col = i / sc, q = i - col * sc, co = c0 + kCols * col + h;
       if (co >= J.ncols) break;
       float t = 0.f;
 #pragma unroll
@@ -816,13 +823,19 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
   // by an ulp, and the next step's ReLU gates with it.  The update is off the critical path of a step anyway.)
   RedJobs jobs;
   memset(&jobs, 0, sizeof(jobs));
+  const int rows = ((B + p.red_splits - 1) / p.red_splits + 7) & ~7;   // <= kRedRows by the choice of red_splits
+  const int nsplit = (B + rows - 1) / rows;
+  // Columns a thread takes of the first layer's weight gradient.  Float rows are two loads for two columns, and the float model's
+  // layers are narrow: one column (batch 1024, 64 wide 86.5 us for the pass, with two 89); bf16 pairs are one (87 and 82 us for the
+  // 4096-sample model's).
+  const int red_cols = p.bf16 ? 2 : 1;
   auto add_job = [&](const void* M, int m_kind, int64_t ldm, int ncols, const void* S, int s_kind, int64_t lds,
                      int s_cols, int64_t out_off) {
     RedJob& J = jobs.job[jobs.njobs++];
     J.M = M; J.m_kind = m_kind; J.ldm = ldm; J.ncols = ncols;
     J.S = S; J.s_kind = s_kind; J.lds = lds; J.s_cols = s_cols;
     J.tile0 = jobs.ntiles; J.part_off = jobs.total; J.out_off = out_off;
-    jobs.ntiles += s_cols == 1 ? (ncols + kRedWide - 1) / kRedWide : (ncols + kRedPairs - 1) / kRedPairs;
+    jobs.ntiles += s_cols == 1 ? (ncols + kRedWide - 1) / kRedWide : (ncols + 32 * red_cols - 1) / (32 * red_cols);
     jobs.total += ncols * s_cols;
   };
 
@@ -943,10 +956,9 @@ ss_status mlp_bwd(const ss_mlp_desc* desc, float* w, void* w_bf16, float* adagra
   float* partial = reinterpret_cast<float*>(ws + p.red_partial);
   if (jobs.njobs > 0) {
     // all batch reductions of the pass in one launch; the update kernel adds the batch slices
-    int rows = ((B + p.red_splits - 1) / p.red_splits + 7) & ~7;   // <= kRedRows by the choice of red_splits
-    const int nsplit = (B + rows - 1) / rows;
     { SS_TIMED("batch_reduce_partial_kernel", cs);
-    launch_dependent(batch_reduce_partial_kernel, dim3(jobs.ntiles, nsplit), 256, 0, cs, jobs, B, rows, partial);
+    launch_dependent(red_cols == 1 ? batch_reduce_partial_kernel<1> : batch_reduce_partial_kernel<2>, dim3(jobs.ntiles, nsplit), 256, 0,
+                     cs, jobs, B, rows, partial);
     }
     SS_LAUNCH_OK();
     for (int j = 0; j < jobs.njobs; ++j)

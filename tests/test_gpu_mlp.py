@@ -113,6 +113,13 @@ def test_mlp_bf16_batches_around_the_row_groups_of_the_reduction(B):
     _check(cfg)
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("width,n_dense,B", [(8, 16, 65), (40, 13, 1025), (72, 1, 129)])
+def test_mlp_first_layer_gradients_of_one_and_two_columns_a_thread(bf16, width, n_dense, B):
+    """Float gradients are summed a column a thread (32 columns a block), bf16 gradients two (64 a block)."""
+    _check(synth.scaled(synth.CONFIGS["tiny"], B=B, T=3, D=16, bottom=(n_dense, width, 16), top=(64, 64, 1), bf16=bf16))
+
+
 def test_mlp_bf16_medium_shapes_reduced_batch():
     # the medium model's layer widths (tensor-core tiles: K = 1728, N = 512) at a batch with a ragged last tile
     cfg = synth.scaled(synth.CONFIGS["medium"], B=328)
