@@ -1926,15 +1926,18 @@ apply_rows_kernel(const int32_t* __restrict__ uniq, const int32_t* __restrict__ 
 template <int G_, int NV_, int KB_, int kMinBlocks_, int KR_> struct WindowShape {
   static constexpr int G = G_, NV = NV_, KB = KB_, kMinBlocks = kMinBlocks_, KR = KR_;
 };
-// By the float4 a row has, rounded up to a power of two.  `few` is for up to kFew windows per SM, about as many as its blocks hold
-// at once: then a window's own rounds are all the time there is, and more lanes or more registers for them are what counts.
-// us of the update half, 26 tables (of 256 floats 10), as it was with `few` throughout (128 floats: one position a batch at 48
-// registers, which spilled) -> now, for 20 000 lookups a table hit once / 66 / 200 times a row, and Zipf 1.2:
+// By the float4 a row has, rounded up to a power of two.  `few` is for up to kFew windows per SM, fewer than its blocks hold at
+// once: then a window's own rounds are all the time there is, and larger batches or more lanes for them are what counts.  Where
+// that takes 128 registers a thread, it is for one block per SM, two of the wider rows: with four, three replicas of an odd-sized
+// model (48 floats, 50 windows per SM) take 109 us a round instead of 102, though the call alone is a tenth faster up to there.
+// us of the update half, 26 tables (of 256 floats 10), with one shape for any number of windows (rows of 128 floats: one position a
+// batch at 48 registers, which spilled) -> now, for 20 000 lookups a table hit once / 66 / 200 times a row, and Zipf 1.2;
+// then 8 windows per SM, uniform ids and 16 lookups a row:
 template <int kQuads> struct WindowShapeFor;
-template <> struct WindowShapeFor<4> {                     // 16 floats 19 / 14 / 20 / 32 (8 blocks 19 / 14 / 20 / 33)
-  static constexpr int kFew = 0;
+template <> struct WindowShapeFor<4> {                     // 16 floats 19 / 14 / 20 / 32 (8 blocks 19 / 14 / 20 / 33); 12 floats 9.9, 7.6 -> 9.4, 7.4
+  static constexpr int kFew = 32;
   using many = WindowShape<4, 1, 4, 7, 0>;
-  using few = many;
+  using few = WindowShape<4, 1, 8, 4, 0>;
 };
 template <> struct WindowShapeFor<8> {                     // 32 floats 29 / 20 / 27 / 39 -> 24 / 17 / 22 / 38, 17 to 31 floats alike;
   static constexpr int kFew = 120;                         // 4000 lookups a table `few` 15, `many` 17
@@ -1942,14 +1945,14 @@ template <> struct WindowShapeFor<8> {                     // 32 floats 29 / 20 
   using few = WindowShape<8, 1, 2, 10, 0>;
 };
 template <> struct WindowShapeFor<16> {                    // 64 floats 47 / 22 / 29 / 55 -> 47 / 22 / 28 / 54, 48 floats 47 / 25 / 31 / 60 ->
-  static constexpr int kFew = 0;                           // 48 / 24 / 30 / 61
+  static constexpr int kFew = 16;                          // 48 / 24 / 30 / 61; 48 floats 14.8, 11.5 -> 12.1, 10.4
   using many = WindowShape<8, 2, 2, 8, 8>;
-  using few = many;
+  using few = WindowShape<8, 2, 4, 4, 0>;
 };
 template <> struct WindowShapeFor<32> {                    // 128 floats 87 / 37 / 39 / 89 -> 85 / 36 / 37 / 85, 100 floats
-  static constexpr int kFew = 0;                           // 92 / 40 / 41 / 101 -> 87 / 37 / 38 / 94
+  static constexpr int kFew = 16;                          // 92 / 40 / 41 / 101 -> 87 / 37 / 38 / 94; 100 floats 18.7, 12.2 -> 12.2, 9.8
   using many = WindowShape<16, 2, 2, 8, 4>;
-  using few = many;
+  using few = WindowShape<16, 2, 4, 4, 0>;
 };
 template <> struct WindowShapeFor<64> {                    // 256 floats 67 / - / - / 77 -> 65 / - / - / 72, 160 floats 63 / - / - / 73 ->
   static constexpr int kFew = 28;                          // 57 / - / - / 65; 20 windows an SM `few` 17 to 20, `many` 18 to 22

@@ -275,7 +275,8 @@ def test_bwd_runs_around_windows_blocks_and_spans(D):
 # the same with as many windows per SM as the fused kernel wants of rows of 129 to 256 floats, and as its forms for many windows
 # want; rows that nobody looks up keep the lookups per row low enough for the fused kernel
 @pytest.mark.parametrize("D,per_sm,spare", [(132, 16, True), (200, 16, True), (256, 16, True), (132, 29, True), (256, 29, True),
-                                            (132, 16, False), (256, 29, False), (20, 121, False), (32, 121, False)])
+                                            (132, 16, False), (256, 29, False), (20, 121, False), (32, 121, False),
+                                            (12, 33, False), (16, 33, False), (48, 17, False), (64, 17, False), (100, 17, False), (128, 17, False)])
 def test_bwd_runs_with_many_windows(D, per_sm, spare):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     lengths = [5] + RUN_LENGTHS * (-(-per_sm * sms * 16 // (2 * sum(RUN_LENGTHS))) + 1)
