@@ -6,10 +6,12 @@
 // wide rows) are issued together so several gathers are in flight per lane.
 //
 // Backward: (1-3) stable LSD radix sort by key t*N+row, unique keys and segment offsets, in one launch: ranges of each
-// table in shared memory, or, for tables too long or too skewed for that, tiled passes over all SMs; (4) the sorted lookups are cut into windows of 16 consecutive positions; a lane group
-// sums the gradients of each run of equal keys inside its window in position order.  A run that
-// lies inside one window is final and is updated at once; a run that crosses a window edge leaves
-// partial sums, added in window order by the group in which it starts, or by a second kernel where the run leaves the block.
+// table in shared memory, or, for tables too long or too skewed for that, tiled passes over all SMs; (4) the sorted lookups are cut
+// into windows of 16 consecutive positions; a lane group sums the gradients of each run of equal keys inside its window in position
+// order.  A run that lies inside one window is final and is updated at once; a run that crosses a window edge leaves partial sums,
+// added in window order by the group in which it starts, or by a second kernel where the run leaves the block or covers more than
+// eight windows.  (Rows of more than 256 floats, and of more than 128 where windows are few or rows popular, are summed in memory
+// and updated by a kernel of their own.)
 // Work per group is the same whatever the skew of the row distribution, and every sum has a fixed
 // association, so results do not depend on scheduling.
 #include <type_traits>
@@ -1337,8 +1339,8 @@ __device__ __forceinline__ bool ws_matches(const int32_t* scalars, int64_t L, ui
 // A lane group owns a window of kWin consecutive sorted positions and adds the gradient rows of each
 // run of equal keys in position order.  A run that lies inside the window is complete: its sum goes
 // to gsum[u].  A run that crosses a window edge leaves a partial sum in the window's slot 0 (run
-// covers the window's first position) or slot 1.  This kernel serves rows wider than 256 floats, and of
-// more than 128 where the windows are few; the others take window_apply_kernel, which also updates the rows.
+// covers the window's first position) or slot 1.  This kernel serves rows wider than 256 floats, and of more than
+// 128 where windows are few or rows popular; the others take window_apply_kernel, which also updates the rows.
 template <int G, int NV>
 __global__ void __launch_bounds__(256)
 window_reduce_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict__ sbag,
@@ -1438,10 +1440,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // structure of a window as 16-bit masks.  A batch of positions requests its gradient rows and, for the runs that end in it, the
 // table rows and states at once; then it adds, and updates a row where a run ends.  A run of up to kShortSpan windows of one
 // block is finished by the group it starts in, so only runs that leave the block, and long ones, are left to the combine kernel.
-// What bounds it is latency and instruction issue together (half of the issue slots, 45 % of the warp slots): rows one after
-// the other as their runs end, and a thread's keys by itself, took 46 us for 26 skewed tables of 21 500 lookups of 64 floats
-// (with the combine kernel 58; now 42 and 51), 100 us for 40 tables of 32 900 of 16 floats (now 84), 16 for 11 of 10 700 of
-// 48 (the same; with the combine kernel 21, now 19).  Additions and steps take two floats an instruction.
+// What bounds it is latency: 40 % of the issue slots, 44 of the warp slots, 27 of DRAM (26 skewed tables of 21 500 lookups of 64
+// floats; 128 floats 43, 46 and 20; 32 floats 41, 47 and 23).  Rows one after the other as their runs end, and a thread's keys by
+// itself, took 46 us for those tables (with the combine kernel 58; now 42 and 50), 100 us for 40 tables of 32 900 of 16 floats (now
+// 84), 16 for 11 of 10 700 of 48 (the same; with the combine kernel 21, now 19).  Additions and steps take two floats an
+// instruction.
 constexpr int kShortSpan = 8;                              // most windows whose parts one lane group adds
 constexpr int kWaThreads = 128;
 
@@ -1752,7 +1755,7 @@ window_apply_kernel(const uint32_t* __restrict__ keys, const int32_t* __restrict
 // block per row, lane group j adds the partials of windows k0+j, k0+j+groups, ... in ascending order and
 // the group sums are then added in group order.  The association is fixed by the
 // segment's position alone (the order of the list does not matter).
-// FUSE (rows of at most 256 floats): the combined sum is not stored; the row is updated here.
+// FUSE (behind window_apply_kernel): the combined sum is not stored; the row is updated here.
 template <int G, int NV, bool FUSE, bool Wide>
 __global__ void __launch_bounds__(256)
 combine_rows_kernel(const int32_t* __restrict__ seg, int32_t* scalars,
@@ -2076,17 +2079,18 @@ __global__ void unique_finish_kernel(const __grid_constant__ SortOut o) { wait_f
 // a call by itself, which runs beside other work (three replicas of 11 tables of 10 700 lookups 104 us a round; 107 with 2750 a
 // range, 121 with 1400 and half of the SMs); down to 1400, up to six ranges on a third of them, where the update waits for the sort
 // in the same call.  One such call alone would take half of the SMs (12 tables of 10 200 lookups: by the rule above 50 us, half 41,
-// a third 41; 20 of 6000 45 / 33 / 35), but several at a time lose more than that: three of 12 tables 62 / 61 / 54, four 72 / 80 / 68,
-// four of 11 64 / 73 / 63, four of 16 of 20 500 116 / 126 / 116.  With eight ranges a table's list is walked too often (3 of 32 800,
-// Zipf 1.2: 71 us, six 66), and two a table are still worth half of the SMs (26 of 5100: 42 us with one, 37).  Blocks without a
-// range cost nothing that could be measured.
+// a third 41), but several at a time lose more than that: three of 12 tables 62 / 61 / 54, four 72 / 80 / 68, four of 11
+// 64 / 73 / 63, four of 16 of 20 500 116 / 126 / 116.  Up to three ranges a table are worth half of the SMs all the same (22 of
+// 25 900, Zipf 1.2: 177 us with two ranges, 147 with three; 26 of 5100 42 with one, 37 with two); four calls at a time lose there
+// (132 -> 143 for 22 of 25 900).  With eight ranges a table's list is walked too often (3 of 32 800, Zipf 1.2: 71 us, six 66).
+// Blocks without a range cost nothing that could be measured.
 static bool plan_bucket_sort(int T, int64_t N, int B, int64_t L, bool waited_for, BucketSort* a, int64_t* blocks, int* nb) {
   const int64_t avg = (L + T - 1) / T;
   if (B > 65535 || avg > 44000) return false;              // bag numbers, plus one, take 16 bits
   int64_t C = (avg + kBsRange - 1) / kBsRange;
   const int64_t least = waited_for ? 1400 : 5500, fine = (avg + least - 1) / least, most = waited_for ? 6 : kBsMaxBuckets;
   int64_t room = num_sms() / (waited_for ? 3 : 4) / T;
-  if (waited_for && room < 2) room = num_sms() / 2 / T;
+  if (waited_for && room < 3) room = num_sms() / 2 / T < 3 ? num_sms() / 2 / T : 3;
   a->per_range = kBsRange;
   if (C < fine && C < room) {
     C = fine < room ? fine : room;

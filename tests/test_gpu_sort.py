@@ -114,7 +114,7 @@ def test_sort_skips_malformed_lookups_in_every_form(B, bag):
 
 
 # the form whose update waits for the sort cuts few tables finer: 1400 lookups a range, up to six ranges, a third of the SMs (half for
-# two ranges a table)
+# up to three ranges a table)
 @pytest.mark.parametrize("T,N,B,bag,rows", [
     (1, 50_000, 1400, 1, UNIFORM), (1, 50_000, 1401, 1, UNIFORM),       # one range, two
     (3, 1000, 700, 16, UNIFORM), (5, 300_007, 1500, 6, HOT_LOW), (1, 5, 2000, 10, UNIFORM),   # six ranges; fewer rows than ranges
