@@ -1440,8 +1440,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // structure of a window as 16-bit masks.  A batch of positions requests its gradient rows and, for the runs that end in it, the
 // table rows and states at once; then it adds, and updates a row where a run ends.  A run of up to kShortSpan windows of one
 // block is finished by the group it starts in, so only runs that leave the block, and long ones, are left to the combine kernel.
-// What bounds it is latency: 40 % of the issue slots, 44 of the warp slots, 27 of DRAM (26 skewed tables of 21 500 lookups of 64
-// floats; 128 floats 43, 46 and 20; 32 floats 41, 47 and 23).  Rows one after the other as their runs end, and a thread's keys by
+// What bounds it is latency: 40 % of the issue slots, 41 of the warp slots, 40 of DRAM (26 skewed tables of 21 500 lookups of 64
+// floats; 128 floats 43, 44 and 44; 32 floats 41, 41 and 27; 256 floats 35, 42 and 44).  Rows one after the other as their runs end, and a thread's keys by
 // itself, took 46 us for those tables (with the combine kernel 58; now 42 and 50), 100 us for 40 tables of 32 900 of 16 floats (now
 // 84), 16 for 11 of 10 700 of 48 (the same; with the combine kernel 21, now 19).  Additions and steps take two floats an
 // instruction.
