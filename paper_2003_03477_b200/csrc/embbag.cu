@@ -2053,7 +2053,7 @@ static void launch_reduce(const BwdPlan& p, char* ws, const uint32_t* keys, int 
   };
   if constexpr (NV == 1) as(std::true_type());
   else if constexpr (NV > 2) as(std::false_type());
-  else if (p.nwin >= kFuseWindows * num_sms() && p.L <= kFuseHits * T * N) as(std::true_type());
+  else if (p.nwin >= kFuseWindows * num_sms() && p.L <= (int64_t)kFuseHits * T * N) as(std::true_type());
   else as(std::false_type());
 }
 
